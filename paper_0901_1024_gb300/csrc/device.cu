@@ -27,6 +27,9 @@ template <int N>
 cudaError_t launch_tc_stage_n(bool rk, const StageArgs& a, int num_sms, cudaStream_t s);
 template <int N>
 cudaError_t launch_tt_stage_n(bool rk, const StageArgs& a, int num_sms, cudaStream_t s);
+template <int N>
+cudaError_t launch_tw_stage_n(bool rk, bool shifted, const StageArgs& a, int num_sms,
+                              cudaStream_t s);
 
 cudaError_t launch_tc_stage(int N, bool rk, const StageArgs& a, int num_sms, cudaStream_t s) {
   switch (N) {
@@ -37,6 +40,17 @@ cudaError_t launch_tc_stage(int N, bool rk, const StageArgs& a, int num_sms, cud
     case 5: return launch_tt_stage_n<5>(rk, a, num_sms, s);
     case 6: return launch_tt_stage_n<6>(rk, a, num_sms, s);
     case 7: return launch_tt_stage_n<7>(rk, a, num_sms, s);
+    default: return cudaErrorInvalidValue;
+  }
+}
+
+// shifted: field chunks off the 16-byte grid (K * Np not a multiple of 4, or an
+// unaligned buffer).
+static cudaError_t launch_tw_stage(int N, bool rk, bool shifted, const StageArgs& a, int num_sms,
+                                   cudaStream_t s) {
+  switch (N) {
+    case 8: return launch_tw_stage_n<8>(rk, shifted, a, num_sms, s);
+    case 9: return launch_tw_stage_n<9>(rk, shifted, a, num_sms, s);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -443,6 +457,7 @@ struct DeviceState {
   double* result = nullptr;
   int egrid = 0;
   void* tcB = nullptr;          // tensor-core B pieces (orders <= kTcMaxOrder)
+  void* twB = nullptr;          // operator stream (orders of tw_order)
   float4* mat = nullptr;        // material records (meshes with materials), in the arena
   bool absorbing = false;       // some boundary face is absorbing
   float* tcgeo = nullptr;       // word-major geometry for the tensor-core stage
@@ -561,8 +576,12 @@ struct OrderOps {
   unsigned char* fmask = nullptr;
   unsigned char* perm = nullptr;
   void* tcB = nullptr;
+  void* twB = nullptr;
   float tc_inv_bscale = 1.f;
 };
+
+// Orders that may run the streamed-operator stage (tw_stage.cuh).
+static bool tw_order(int N) { return N >= 8; }
 
 static std::mutex g_ops_mutex;
 static std::map<std::pair<int, int>, OrderOps> g_ops;
@@ -667,6 +686,41 @@ static int order_ops(const dg_mesh* m, int dev, OrderOps& out, std::string& err)
       }
     if ((rc = upload(reinterpret_cast<__half**>(&o.tcB), P, err))) return rc;
   }
+  if (tw_order(m->N)) {
+    // The streamed operator: step st of 16 K columns is node block st / 3 of
+    // Dr, Ds or Dt (st % 3), after those face-node block st - 3 JB of LIFT; zero
+    // padded, scaled by 2^p, hi then lo, [2 chunks of 8 columns][NN nodes].
+    const int N = m->N, NN = dgdev::tw_nn(N), JB = dgdev::tw_jblocks(N), KS = dgdev::tw_steps(N);
+    auto value = [&](int n, int st, int kk) -> double {
+      if (n >= Np) return 0.0;
+      if (st < 3 * JB) {
+        const int j = 16 * (st / 3) + kk, mu = st % 3;
+        const std::vector<double>& Dm = mu == 0 ? m->ops.Dr : mu == 1 ? m->ops.Ds : m->ops.Dt;
+        return j < Np ? Dm[n * Np + j] : 0.0;
+      }
+      const int f = 16 * (st - 3 * JB) + kk;
+      return f < NF ? m->ops.LIFT[n * NF + f] : 0.0;
+    };
+    double mx = 0.0;
+    for (int n = 0; n < Np; ++n)
+      for (int st = 0; st < KS; ++st)
+        for (int kk = 0; kk < 16; ++kk) mx = std::max(mx, std::fabs(value(n, st, kk)));
+    const double sB = std::ldexp(1.0, static_cast<int>(std::floor(std::log2(16384.0 / mx))));
+    o.tc_inv_bscale = static_cast<float>(1.0 / sB);
+    std::vector<__half> P(static_cast<size_t>(dgdev::tw_b_bytes(N)) / 2);
+    for (int st = 0; st < KS; ++st)
+      for (int n = 0; n < NN; ++n)
+        for (int kk = 0; kk < 16; ++kk) {
+          // the low piece from the FP64 operator: its FP32 rounding is not split too
+          const double x = value(n, st, kk) * sB;
+          const __half hi = __float2half_rn(static_cast<float>(x));
+          const __half lo = __double2half(x - static_cast<double>(__half2float(hi)));
+          const size_t off = ((static_cast<size_t>(st) * 4 + kk / 8) * NN + n) * 8 + kk % 8;
+          P[off] = hi;
+          P[off + static_cast<size_t>(2) * NN * 8] = lo;
+        }
+    if ((rc = upload(reinterpret_cast<__half**>(&o.twB), P, err))) return rc;
+  }
   g_ops[{dev, m->N}] = o;
   out = o;
   return DG_OK;
@@ -700,19 +754,19 @@ int ensure_device(dg_mesh* m, std::string& err) {
   d->fmask = ops.fmask;
   d->perm = ops.perm;
   d->tcB = ops.tcB;
+  d->twB = ops.twB;
   d->tc_inv_bscale = ops.tc_inv_bscale;
   const int64_t K = m->K;
   const int Nfp = d->Nfp, NF = 4 * Nfp;
-  const bool tc = d->N <= dgdev::kTcMaxOrder;
   const int E = dgdev::tc_tile_elems(d->N);
   const int64_t ntiles = (K + E - 1) / E;
-  d->tc_geo_stride = tc ? dgdev::tc_geo_floats(d->N) : 0;
+  d->tc_geo_stride = dgdev::tc_geo_floats(d->N);
   d->egrid = dgdev::energy_grid(d->num_sms);
   // arena layout (bytes, each part 256-byte aligned)
   auto up = [](size_t x) { return (x + 255) & ~size_t(255); };
   const size_t geo_b = static_cast<size_t>(K) * dgdev::kGeoWords * 4;
   const size_t mat_b = m->eps.empty() ? 0 : static_cast<size_t>(K) * dgdev::kMatVecs * 16;
-  const size_t tcg_b = tc ? static_cast<size_t>(ntiles) * d->tc_geo_stride * 4 : 0;
+  const size_t tcg_b = static_cast<size_t>(ntiles) * d->tc_geo_stride * 4;
   const size_t o_mat = up(geo_b), o_tcg = o_mat + up(mat_b), o_part = o_tcg + up(tcg_b);
   const size_t o_res = o_part + up(sizeof(double) * d->egrid), o_stat = o_res + 256;
   const size_t total = o_stat + 256;
@@ -755,7 +809,7 @@ int ensure_device(dg_mesh* m, std::string& err) {
       }
     }
   }
-  if (tc) {
+  {
     // tiled geometry, one contiguous block per tile: word-major [kTcGeoWords][E]
     // (record words {0..8 metric, 10 codes, 12..27 faces, 28..31 neighbours} ->
     // words {0..8, 9, 10..25, 26..29}), then one byte per face node (e, m):
@@ -782,31 +836,44 @@ int ensure_device(dg_mesh* m, std::string& err) {
   DG_CUDA(cudaMemset(base + o_stat, 0, 256), "cudaMemset");
   d->geo = reinterpret_cast<float4*>(base);
   d->mat = mat_b ? reinterpret_cast<float4*>(base + o_mat) : nullptr;
-  d->tcgeo = tc ? reinterpret_cast<float*>(base + o_tcg) : nullptr;
+  d->tcgeo = reinterpret_cast<float*>(base + o_tcg);
   d->partials = reinterpret_cast<double*>(base + o_part);
   d->result = reinterpret_cast<double*>(base + o_res);
   d->status = reinterpret_cast<int*>(base + o_stat);
   return DG_OK;
 }
 
-// Tensor cores for orders 2..kTcMaxOrder (and 1 on request) unless the CUDA-core
-// path is forced.
-// The tensor-core kernel moves whole tiles with bulk copies, which need every
-// field chunk 16-byte aligned: (K * Np) % 4 == 0 and 16-byte aligned buffers.
-static bool use_tc(const dg_mesh* m, std::initializer_list<const void*> bufs) {
-  if (m->stage_impl == DG_STAGE_FP32 || m->N > dgdev::kTcMaxOrder) return false;
-  // at N = 1 (Np = 4) the FP32 kernel is faster unless tensor cores are asked for
-  if (m->stage_impl == DG_STAGE_AUTO && m->N == 1) return false;
-  if ((m->K * m->ops.Np) % 4 != 0) return false;
-  for (const void* p : bufs)
-    if (reinterpret_cast<uintptr_t>(p) % 16 != 0) return false;
-  return true;
+// The kernel family of a stage call.
+enum class Path { fp32, tc, tw, tw_shifted };
+
+// DG_STAGE_TC and orders 2..7 of DG_STAGE_AUTO: the tensor-core stages of
+// tc_stage.cuh and tc_stage_t.cuh, which move whole tiles with bulk copies and need
+// every field chunk 16-byte aligned ((K * Np) % 4 == 0 and 16-byte aligned buffers).
+// DG_STAGE_AUTO at orders 8 and 9: the streamed-operator tensor-core stage, shifted
+// where chunks are off the 16-byte grid.  Everything else: FP32 CUDA cores (N = 1,
+// Np = 4, is faster there than on the tensor cores).
+static Path stage_path(const dg_mesh* m, std::initializer_list<const void*> bufs) {
+  if (m->stage_impl == DG_STAGE_FP32) return Path::fp32;
+  bool aligned = (m->K * m->ops.Np) % 4 == 0;
+  for (const void* p : bufs) aligned = aligned && reinterpret_cast<uintptr_t>(p) % 16 == 0;
+  if (m->stage_impl == DG_STAGE_AUTO) {
+    if (m->N == 1) return Path::fp32;
+    if (tw_order(m->N))
+      return aligned ? Path::tw : m->ops.Np % 4 != 0 ? Path::tw_shifted : Path::fp32;
+  }
+  return m->N <= dgdev::kTcMaxOrder && aligned ? Path::tc : Path::fp32;
 }
 
-static dgdev::StageArgs stage_args(dg_mesh* m, bool tc) {
+static int stage_tile(const dg_mesh* m, Path p) {
+  return p == Path::fp32 ? dgdev::stage_tile_elems(m->N, m->stage_shape)
+                         : dgdev::tc_tile_elems(m->N);
+}
+
+static dgdev::StageArgs stage_args(dg_mesh* m, Path p) {
   DeviceState* d = m->dev;
   dgdev::StageArgs a{};
   a.tcB = d->tcB;
+  a.twB = d->twB;
   a.tcgeo = d->tcgeo;
   a.tc_geo_stride = d->tc_geo_stride;
   a.tc_inv_bscale = d->tc_inv_bscale;
@@ -820,24 +887,32 @@ static dgdev::StageArgs stage_args(dg_mesh* m, bool tc) {
   a.perm = d->perm;
   a.K = static_cast<int>(d->K);
   a.alpha = static_cast<float>(m->alpha);
-  const int E = tc ? dgdev::tc_tile_elems(d->N) : dgdev::stage_tile_elems(d->N, m->stage_shape);
+  const int E = stage_tile(m, p);
   a.num_tiles = static_cast<int>((d->K + E - 1) / E);
   return a;
+}
+
+static cudaError_t launch_path(const dg_mesh* m, Path p, bool rk, const dgdev::StageArgs& a,
+                               cudaStream_t s) {
+  const int sms = m->dev->num_sms;
+  switch (p) {
+    case Path::tc: return dgdev::launch_tc_stage(m->N, rk, a, sms, s);
+    case Path::tw: return dgdev::launch_tw_stage(m->N, rk, false, a, sms, s);
+    case Path::tw_shifted: return dgdev::launch_tw_stage(m->N, rk, true, a, sms, s);
+    default: return dgdev::launch_stage(m->N, rk, a, sms, s, m->stage_shape);
+  }
 }
 
 int device_rhs(dg_mesh* m, const float* u, float* rhs, void* stream, std::string& err) {
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   int rc = ensure_device(m, err);
   if (rc) return rc;
-  const bool tc = use_tc(m, {u, rhs});
-  dgdev::StageArgs a = stage_args(m, tc);
+  const Path p = stage_path(m, {u, rhs});
+  dgdev::StageArgs a = stage_args(m, p);
   a.u_in = u;
   a.rhs = rhs;
-  DG_CUDA(traced(m, s, tc ? 5 : 1, [&] {
-            return tc ? dgdev::launch_tc_stage(m->N, false, a, m->dev->num_sms, s)
-                             : dgdev::launch_stage(m->N, false, a, m->dev->num_sms, s,
-                                                   m->stage_shape);
-          }), "stage kernel launch");
+  DG_CUDA(traced(m, s, p == Path::fp32 ? 1 : 5, [&] { return launch_path(m, p, false, a, s); }),
+          "stage kernel launch");
   m->last_launches = 1;
   return DG_OK;
 }
@@ -858,8 +933,8 @@ static int step_impl(dg_mesh* m, float* u, float* res, double dt, int nsteps, cu
   DeviceState* d = m->dev;
   const size_t n = static_cast<size_t>(6) * d->K * d->Np;
   if (!d->u_work) DG_CUDA(cudaMalloc(&d->u_work, n * sizeof(float)), "cudaMalloc work state");
-  const bool tc = use_tc(m, {u, res, d->u_work});
-  dgdev::StageArgs a = stage_args(m, tc);
+  const Path p = stage_path(m, {u, res, d->u_work});
+  dgdev::StageArgs a = stage_args(m, p);
   a.res = res;
   a.dt = static_cast<float>(dt);
   const float* src = u;
@@ -871,10 +946,8 @@ static int step_impl(dg_mesh* m, float* u, float* res, double dt, int nsteps, cu
       a.u_out = dst;
       a.a = static_cast<float>(kRkA[i]);
       a.b = static_cast<float>(kRkB[i]);
-      DG_CUDA(traced(m, s, tc ? 4 : 0, [&] {
-                return tc ? dgdev::launch_tc_stage(m->N, true, a, d->num_sms, s)
-                          : dgdev::launch_stage(m->N, true, a, d->num_sms, s, m->stage_shape);
-              }), "stage kernel launch");
+      DG_CUDA(traced(m, s, p == Path::fp32 ? 0 : 4, [&] { return launch_path(m, p, true, a, s); }),
+              "stage kernel launch");
       ++launches;
       float* nsrc = dst;
       dst = const_cast<float*>(src);
@@ -891,8 +964,7 @@ int device_stage_tile(dg_mesh* m, const float* u_in, const float* u_out, const f
                       int* tile, std::string& err) {
   int rc = ensure_device(m, err);
   if (rc) return rc;
-  *tile = use_tc(m, {u_in, u_out, res}) ? dgdev::tc_tile_elems(m->N)
-                                        : dgdev::stage_tile_elems(m->N, m->stage_shape);
+  *tile = stage_tile(m, stage_path(m, {u_in, u_out, res}));
   return DG_OK;
 }
 
@@ -901,11 +973,10 @@ int device_stage(dg_mesh* m, const float* u_in, float* u_out, float* res, int st
   int rc = ensure_device(m, err);
   if (rc) return rc;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  DeviceState* d = m->dev;
-  const bool tc = use_tc(m, {u_in, u_out, res});
-  dgdev::StageArgs a = stage_args(m, tc);
+  const Path p = stage_path(m, {u_in, u_out, res});
+  dgdev::StageArgs a = stage_args(m, p);
   if (k1 >= 0) {                        // elements [k0, k1): whole tiles of the kernel that runs
-    const int E = tc ? dgdev::tc_tile_elems(m->N) : dgdev::stage_tile_elems(m->N, m->stage_shape);
+    const int E = stage_tile(m, p);
     if (k0 < 0 || k1 <= k0 || k1 > m->K || k0 % E != 0 || (k1 % E != 0 && k1 != m->K)) {
       err = "the element range must be [k0, k1) with k0 and k1 multiples of the stage's tile of " +
             std::to_string(E) + " tetrahedra (or k1 = K), 0 <= k0 < k1 <= K";
@@ -921,10 +992,8 @@ int device_stage(dg_mesh* m, const float* u_in, float* u_out, float* res, int st
   a.dt_elem = dt_elem;
   a.a = static_cast<float>(kRkA[stage]);
   a.b = static_cast<float>(kRkB[stage]);
-  DG_CUDA(traced(m, s, tc ? 4 : 0, [&] {
-            return tc ? dgdev::launch_tc_stage(m->N, true, a, d->num_sms, s)
-                      : dgdev::launch_stage(m->N, true, a, d->num_sms, s, m->stage_shape);
-          }), "stage kernel launch");
+  DG_CUDA(traced(m, s, p == Path::fp32 ? 0 : 4, [&] { return launch_path(m, p, true, a, s); }),
+          "stage kernel launch");
   m->last_launches = 1;
   return DG_OK;
 }
@@ -971,7 +1040,7 @@ int device_stage_multi(dg_mesh* const* ms, int n, const float* const* u_in, floa
       err = "every mesh of one call must be on the same device";
       return DG_ERR_ARG;
     }
-    if (use_tc(ms[i], {u_in[i], u_out[i], res[i]})) fam[i] = ms[i]->N <= 4 ? 1 : ms[i]->N <= 6 ? 2 : 0;
+    if (stage_path(ms[i], {u_in[i], u_out[i], res[i]}) == Path::tc) fam[i] = ms[i]->N <= 4 ? 1 : ms[i]->N <= 6 ? 2 : 0;
   }
   for (int i = 0; i < n; ++i)
     if (fam[i] == 0) {
@@ -994,7 +1063,7 @@ int device_stage_multi(dg_mesh* const* ms, int n, const float* const* u_in, floa
       int64_t all = 0;
       for (size_t g = 0; g < ng; ++g) {
         const int i = idx[c0 + g];
-        dgdev::StageArgs a = stage_args(ms[i], true);
+        dgdev::StageArgs a = stage_args(ms[i], Path::tc);
         a.u_in = u_in[i];
         a.u_out = u_out[i];
         a.res = res[i];
