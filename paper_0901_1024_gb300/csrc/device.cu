@@ -75,296 +75,153 @@ cudaError_t launch_stage(int N, bool rk, const StageArgs& a, int num_sms, cudaSt
 // E = 1/2 sum_k J_k sum_c u_kc^T M u_kc.  Each block writes one FP64 partial
 // (its threads' sums, added in a fixed order) and a one-warp kernel adds the
 // partials in a fixed order, so the result is deterministic.
-constexpr int kEnergyThreads = 256;
-constexpr int kEnergyRows = 128;      // field rows (c, k) per block pass, row kernel
-
-// Row kernel (orders 1, 2, 3, 5): a block stages 128 consecutive field rows (c, k) in shared
-// memory per pass (row stride NP | 1: conflict-free), thread r then keeps row r
-// in registers and forms u^T M u from M's rows, read as broadcast 16-byte loads.
-// The rows arrive by 4-byte cp.async copies (a pass's copies are all in flight
-// at once, coalesced); where shared memory allows four blocks per SM the next
-// pass's copies are issued before the current pass is computed.
-template <int NP>
-struct EnergyRowsShape {
-  static constexpr int NP4 = (NP + 3) & ~3, RS = NP | 1;
-  // Up to 56 nodes M is used as its upper triangle (M symmetric:
-  // u^T M u = sum_i u_i (M_ii u_i + 2 sum_{j>i} M_ij u_j)), row i holding
-  // M_ii, 2 M_i,i+1, ..., 2 M_i,NP-1 from a 16-byte boundary; above that the
-  // full matrix, row-padded to NP4.
-  static constexpr bool TRI = NP <= 56;
-  __host__ __device__ static constexpr int tri_off(int i) {
+//
+// With T_ji = M_ii, 2 M_ij for j > i, 0 for j < i (M symmetric), u^T M u =
+// sum_i u_i s_i, s_i = sum_{j >= i} T_ji u_j: a small triangular matrix product over
+// all rows (c, k).  It is bound by FP32 arithmetic from N = 6 on (N = 9: 3.8 GFLOP on
+// 1.7e7 unknowns, 48 us at the FP32 peak, against 10 us to read the fields) and by
+// reading them below.  So it runs as a register-tiled product: blocks of 32 outputs i
+// (the triangle is skipped at that grain), a warp forms 32 rows x 32 outputs of one
+// block, a lane 8 rows x 4 outputs, and 4 columns j cost it 12 16-byte shared loads for
+// 128 multiply-adds (the row-per-thread kernels before it loaded 32 bytes of M for 8 or
+// 16, with one to eight warps an SM).  T and a pass of rows sit in shared memory; the
+// (row set, output block) tasks go to the warps longest first, every second round in
+// reverse, which balances the triangle.  FP32 products and row sums, FP64 sums of the
+// weighted rows.  A whole dg_energy call on ~1.7e7 unknowns (35 us of it launches, copy
+// and synchronisation), before and after: N = 9 1184 -> 160 us, N = 8 515 -> 127, N = 7
+// 207 -> 98, N = 6 122 -> 86, N = 5 110 -> 76, N = 4 83 -> 76, N = 3 84 -> 64.  The
+// Jacobians are read from an array of their own: from the 128-byte element records each
+// row would fetch a whole sector for one word.
+template <int N> struct EnergyShape {
+  static constexpr int NP = (N + 1) * (N + 2) * (N + 3) / 6;
+  static constexpr int NP4 = (NP + 3) & ~3;            // row stride: 4 rows of a warp never share banks
+  static constexpr int NB = (NP + 31) / 32;            // output blocks
+  static constexpr int RSETS = N == 8 ? 2 : 4;         // row sets of 32 per pass
+  static constexpr int ROWS = 32 * RSETS;
+  static constexpr int WARPS = N == 9 ? 14 : N == 8 ? 6 : N >= 6 ? 8 : 4;
+  static constexpr int THREADS = 32 * WARPS, MIN_BLOCKS = N == 9 ? 1 : N >= 6 ? 2 : 4;
+  __host__ __device__ static constexpr int t_off(int ob) {   // first float of output block ob
     int o = 0;
-    for (int r = 0; r < i; ++r) o += (NP - r + 3) & ~3;
+    for (int b = 0; b < ob; ++b) o += (NP4 - 32 * b) * 32;
     return o;
   }
-  static constexpr int M_FLOATS = TRI ? tri_off(NP) : NP * NP4, U_FLOATS = kEnergyRows * RS;
-  static constexpr int NBUF = (M_FLOATS + 2 * U_FLOATS) * 4 <= 56 * 1024 ? 2 : 1;
-  static constexpr int BYTES = (M_FLOATS + NBUF * U_FLOATS) * 4;
+  static constexpr int T_FLOATS = t_off(NB);           // [block][j - 32 block][32 outputs]
+  static constexpr int BYTES = (T_FLOATS + ROWS * NP4) * 4 + ROWS * 12;
+  static_assert(NP4 % 32 % 16 != 0, "bank-conflict-free row reads");
+  static_assert(BYTES <= 227 * 1024, "shared memory");
 };
 
-template <int NP>
-__global__ void __launch_bounds__(kEnergyRows) energy_rows_kernel(const EnergyArgs A) {
-  using S = EnergyRowsShape<NP>;
-  constexpr int NP4 = S::NP4, RS = S::RS, NBUF = S::NBUF;
+template <int N, bool VEC>
+__global__ void __launch_bounds__(EnergyShape<N>::THREADS, EnergyShape<N>::MIN_BLOCKS)
+energy_tile_kernel(const EnergyArgs A) {
+  using S = EnergyShape<N>;
+  constexpr int NP = S::NP, NP4 = S::NP4, NB = S::NB, ROWS = S::ROWS, TH = S::THREADS;
   extern __shared__ __align__(16) float esm[];
-  float* sM = esm;                       // [NP][NP4], zero padded
-  float* sU = esm + S::M_FLOATS;         // [NBUF][kEnergyRows][RS]
-  __shared__ int64_t sRow[NBUF][kEnergyRows];
-  if constexpr (S::TRI) {
-    for (int r = 0; r < NP; ++r)         // row r: columns r .. NP-1, zero padded
-      for (int c = threadIdx.x; c < ((NP - r + 3) & ~3); c += kEnergyRows)
-        sM[S::tri_off(r) + c] = r + c < NP ? (c ? 2.f : 1.f) * __ldg(A.M + r * NP + r + c) : 0.f;
-  } else {
-    for (int i = threadIdx.x; i < NP * NP4; i += kEnergyRows) {
-      const int r = i / NP4, c = i - r * NP4;
-      sM[i] = c < NP ? __ldg(A.M + r * NP + c) : 0.f;
-    }
-  }
-  // rows (c, k) for k0 <= k < k1, numbered c * Kr + (k - k0); pass p of this
-  // block covers rows [r0(p), r0(p) + 128)
-  const int64_t Kr = A.k1 - A.k0, rows = 6 * Kr;
-  const int64_t first = int64_t(blockIdx.x) * kEnergyRows, stride = int64_t(gridDim.x) * kEnergyRows;
-  // thread t's row of a pass: its global offset (published for the copies);
-  // returns its weight J_k (times eps_k for E rows, mu_k for H rows with
-  // materials), loaded a pass ahead with two buffers (> 0), or -1 for no row
-  auto row_of = [&](int64_t r0, int b) -> float {
-    const int64_t g = r0 + threadIdx.x;
-    if (g >= rows) return -1.f;
-    const int64_t c = g / Kr, k = A.k0 + (g - c * Kr);
-    sRow[b][threadIdx.x] = (c * A.K + k) * NP;
-    const float J = __ldg(reinterpret_cast<const float*>(A.geo) + k * kGeoWords + 9);
-    if (!A.mat) return J;
-    const float4 w = __ldg(A.mat + k * kMatVecs);
-    return J * (c < 3 ? w.z : w.w);
-  };
-  auto issue = [&](int64_t r0, int b) {
-    if (r0 < rows) {
-      const int nr = int(rows - r0 < kEnergyRows ? rows - r0 : kEnergyRows);
-      float* dst = sU + b * S::U_FLOATS;
-      for (int i = threadIdx.x; i < nr * NP; i += kEnergyRows) {
-        const int r = i / NP, j = i - r * NP;
-        tc::cp_async4(dst + r * RS + j, A.u + sRow[b][r] + j);
-      }
-    }
-    tc::cp_async_commit();               // possibly empty: keeps the group count uniform
-  };
+  float* sT = esm;
+  float* sU = esm + S::T_FLOATS;                       // [ROWS][NP4]
+  int64_t* sRow = reinterpret_cast<int64_t*>(sU + ROWS * NP4);
+  float* sW = reinterpret_cast<float*>(sRow + ROWS);
+  const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31, rg = lane >> 3, og = lane & 7;
+  for (int i = tid; i < S::T_FLOATS / 4; i += TH)
+    tc::cp_async16(reinterpret_cast<float4*>(sT) + i, reinterpret_cast<const float4*>(A.T) + i);
+  if constexpr (NP4 != NP)                             // padding columns stay zero
+    for (int i = tid; i < ROWS * (NP4 - NP); i += TH)
+      sU[i / (NP4 - NP) * NP4 + NP + i % (NP4 - NP)] = 0.f;
+  const unsigned Kr = unsigned(A.k1 - A.k0), rows = 6u * Kr;   // rows (c, k): c Kr + (k - k0)
   double acc = 0.0;
-  float J_cur = -1.f;
-  if constexpr (NBUF == 2) {
-    J_cur = row_of(first, 0);
+  for (unsigned r0 = blockIdx.x * ROWS; r0 < rows; r0 += gridDim.x * ROWS) {
+    const int nr = int(min(rows - r0, unsigned(ROWS)));
+    __syncthreads();                                   // the previous pass is consumed
+    for (int i = tid; i < nr; i += TH) {
+      const unsigned g = r0 + i, c = g / Kr;
+      const int64_t k = A.k0 + int64_t(g - c * Kr);
+      sRow[i] = (int64_t(c) * A.K + k) * NP;
+      float wgt = __ldg(A.J + k);
+      if (A.mat) {
+        const float4 m = __ldg(A.mat + k * kMatVecs);
+        wgt *= c < 3 ? m.z : m.w;
+      }
+      sW[i] = wgt;                                     // J_k (times eps_k or mu_k)
+    }
     __syncthreads();
-    issue(first, 0);
-  }
-  for (int p = 0;; ++p) {
-    const int64_t r0 = first + p * stride;
-    const int b = NBUF == 2 ? (p & 1) : 0;
-    float J_next = -1.f;
-    // row offsets of the pass to issue (the next one with two buffers, else
-    // this one); its buffer was last read before the previous barrier
-    if constexpr (NBUF == 2) {
-      if (r0 + stride < rows) J_next = row_of(r0 + stride, b ^ 1);
+    if constexpr (VEC) {                               // whole 16-byte words
+      for (int i = tid; i < nr * (NP / 4); i += TH) {
+        const int r = i / (NP / 4), q = i - r * (NP / 4);
+        tc::cp_async16(reinterpret_cast<float4*>(sU + r * NP4) + q,
+                       reinterpret_cast<const float4*>(A.u + sRow[r]) + q);
+      }
     } else {
-      if (r0 < rows) J_cur = row_of(r0, 0);
-    }
-    __syncthreads();                     // offsets visible; the previous pass is consumed
-    if constexpr (NBUF == 2) issue(r0 + stride, b ^ 1);
-    else issue(r0, 0);
-    tc::cp_async_wait_group<NBUF - 1>(); // this thread's copies of pass p have landed
-    __syncthreads();                     // everyone's have
-    if (r0 >= rows) break;
-    const float* su = sU + b * S::U_FLOATS + threadIdx.x * RS;
-    if (J_cur >= 0.f) {
-      float u[NP4];
-#pragma unroll
-      for (int j = 0; j < NP4; ++j) u[j] = j < NP ? su[j] : 0.f;
-      float e = 0.f;
-      if constexpr (S::TRI) {
-#pragma unroll
-        for (int i = 0; i < NP; ++i) {
-          const float4* Mi = reinterpret_cast<const float4*>(sM + S::tri_off(i));
-          float s0 = 0.f, s1 = 0.f;
-#pragma unroll
-          for (int q = 0; q < (NP - i + 3) / 4; ++q) {
-            const float4 m4 = Mi[q];
-            const int j = i + 4 * q;
-            s0 = fmaf(m4.x, u[j], s0);
-            if (j + 1 < NP) s1 = fmaf(m4.y, u[j + 1], s1);
-            if (j + 2 < NP) s0 = fmaf(m4.z, u[j + 2], s0);
-            if (j + 3 < NP) s1 = fmaf(m4.w, u[j + 3], s1);
-          }
-          e = fmaf(u[i], s0 + s1, e);
-        }
-      } else {
-#pragma unroll 1
-        for (int i = 0; i < NP; ++i) {
-          const float4* Mi = reinterpret_cast<const float4*>(sM + i * NP4);
-          float s0 = 0.f, s1 = 0.f;        // two chains for instruction-level parallelism
-#pragma unroll
-          for (int j4 = 0; j4 < NP4 / 4; ++j4) {
-            const float4 m4 = Mi[j4];
-            s0 = fmaf(m4.x, u[4 * j4], s0);
-            s1 = fmaf(m4.y, u[4 * j4 + 1], s1);
-            s0 = fmaf(m4.z, u[4 * j4 + 2], s0);
-            s1 = fmaf(m4.w, u[4 * j4 + 3], s1);
-          }
-          e = fmaf(su[i], s0 + s1, e);
-        }
+      for (int i = tid; i < nr * NP; i += TH) {
+        const int r = i / NP, j = i - r * NP;
+        tc::cp_async4(sU + r * NP4 + j, A.u + sRow[r] + j);
       }
-      acc += double(J_cur) * double(e);
-    }
-    if constexpr (NBUF == 2) J_cur = J_next;
-  }
-  tc::cp_async_wait_all();
-  __shared__ double sw[kEnergyRows / 32];
-#pragma unroll
-  for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-  if ((threadIdx.x & 31) == 0) sw[threadIdx.x >> 5] = acc;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double t = 0.0;
-    for (int w = 0; w < kEnergyRows / 32; ++w) t += sw[w];
-    A.partials[blockIdx.x] = t;
-  }
-}
-
-// Orders 4 and 6..9: M (symmetric) in shared memory as its weighted upper triangle,
-// T_ji = M_ij for j = i, 2 M_ij for j > i, 0 below (row j padded to NP8 floats),
-// so u^T M u = sum_i u_i s_i with s_i = sum_{j >= i} T_ji u_j.  Each thread takes
-// RPT field rows (c, k) of a pass, staged by 4-byte cp.async copies with an odd
-// row stride (conflict-free 4-byte reads), and forms s_i for 8 outputs i0..i0+7
-// at a time over j >= i0 (row j of T read as two broadcast 16-byte loads, used
-// for all RPT rows of the thread), then e += sum_i u_i s_i.  FP32 products,
-// FP64 sums of the weighted rows.
-template <int NP, int THREADS, int RPT>
-struct EnergyWideShape {
-  static constexpr int NP8 = (NP + 7) & ~7, RS = NP | 1, ROWS = THREADS * RPT;
-  static constexpr int BYTES = (NP * NP8 + ROWS * RS) * 4;
-  static_assert(BYTES <= 226 * 1024, "shared memory");
-};
-
-template <int NP, int THREADS, int RPT>
-__global__ void __launch_bounds__(THREADS) energy_wide_kernel(const EnergyArgs A) {
-  using S = EnergyWideShape<NP, THREADS, RPT>;
-  constexpr int NP8 = S::NP8, RS = S::RS, ROWS = S::ROWS;
-  extern __shared__ __align__(16) float esm[];
-  float* sM = esm;                       // T: [NP][NP8], zero padded
-  float* sU = esm + NP * NP8;            // [ROWS][RS]
-  __shared__ int64_t sRow[ROWS];
-  for (int i = threadIdx.x; i < NP * NP8; i += THREADS) {
-    const int r = i / NP8, c = i - r * NP8;              // T_rc
-    sM[i] = c < NP && r >= c ? (r > c ? 2.f : 1.f) * __ldg(A.M + r * NP + c) : 0.f;
-  }
-  const int64_t Kr = A.k1 - A.k0, rows = 6 * Kr;
-  double acc = 0.0;
-  for (int64_t r0 = int64_t(blockIdx.x) * ROWS; r0 < rows; r0 += int64_t(gridDim.x) * ROWS) {
-    float w[RPT];                        // J_k (times eps_k or mu_k), or 0: no row
-#pragma unroll
-    for (int q = 0; q < RPT; ++q) {
-      const int lr = threadIdx.x + q * THREADS;
-      const int64_t g = r0 + lr;
-      w[q] = 0.f;
-      if (g < rows) {
-        const int64_t c = g / Kr, k = A.k0 + (g - c * Kr);
-        sRow[lr] = (c * A.K + k) * NP;
-        const float J = __ldg(reinterpret_cast<const float*>(A.geo) + k * kGeoWords + 9);
-        w[q] = J;
-        if (A.mat) {
-          const float4 m = __ldg(A.mat + k * kMatVecs);
-          w[q] = J * (c < 3 ? m.z : m.w);
-        }
-      }
-    }
-    __syncthreads();                     // row offsets visible; the previous pass is consumed
-    const int nr = int(rows - r0 < ROWS ? rows - r0 : ROWS);
-    for (int i = threadIdx.x; i < nr * NP; i += THREADS) {
-      const int r = i / NP, j = i - r * NP;
-      tc::cp_async4(sU + r * RS + j, A.u + sRow[r] + j);
     }
     tc::cp_async_commit();
     tc::cp_async_wait_all();
     __syncthreads();
-    if (threadIdx.x < nr) {
-      const float* u0 = sU + threadIdx.x * RS;
-      float e[RPT];
-#pragma unroll
-      for (int q = 0; q < RPT; ++q) e[q] = 0.f;
 #pragma unroll 1
-      for (int i0 = 0; i0 < NP; i0 += 8) {
-        float sacc[RPT][8];
+    for (int round = 0; round * S::WARPS < NB * S::RSETS; ++round) {
+      const int task = round * S::WARPS + (round & 1 ? S::WARPS - 1 - warp : warp);
+      if (task >= NB * S::RSETS) continue;
+      const int ob = task / S::RSETS, row0 = (task - ob * S::RSETS) * 32 + rg;   // rows row0 + 4 i
+      if (row0 - rg >= nr) continue;
+      const float* u0 = sU + row0 * NP4;
+      const float* t0 = sT + 16 * ob * (2 * NP4 - 32 * (ob - 1)) + og * 4;       // t_off(ob)
+      float s[8][4];
 #pragma unroll
-        for (int q = 0; q < RPT; ++q)
+      for (int i = 0; i < 8; ++i)
 #pragma unroll
-          for (int ii = 0; ii < 8; ++ii) sacc[q][ii] = 0.f;
-#pragma unroll 4
-        for (int j = i0; j < NP; ++j) {
-          const float4 m0 = *reinterpret_cast<const float4*>(sM + j * NP8 + i0);
-          const float4 m1 = *reinterpret_cast<const float4*>(sM + j * NP8 + i0 + 4);
+        for (int x = 0; x < 4; ++x) s[i][x] = 0.f;
+#pragma unroll 1
+      for (int j = 32 * ob; j < NP4; j += 4) {
+        float4 t[4];
 #pragma unroll
-          for (int q = 0; q < RPT; ++q) {
-            const float uj = u0[q * THREADS * RS + j];
-            sacc[q][0] = fmaf(m0.x, uj, sacc[q][0]);
-            sacc[q][1] = fmaf(m0.y, uj, sacc[q][1]);
-            sacc[q][2] = fmaf(m0.z, uj, sacc[q][2]);
-            sacc[q][3] = fmaf(m0.w, uj, sacc[q][3]);
-            sacc[q][4] = fmaf(m1.x, uj, sacc[q][4]);
-            sacc[q][5] = fmaf(m1.y, uj, sacc[q][5]);
-            sacc[q][6] = fmaf(m1.z, uj, sacc[q][6]);
-            sacc[q][7] = fmaf(m1.w, uj, sacc[q][7]);
+        for (int q = 0; q < 4; ++q) t[q] = *reinterpret_cast<const float4*>(t0 + (j - 32 * ob + q) * 32);
+#pragma unroll
+        for (int i = 0; i < 8; ++i) {
+          const float4 u = *reinterpret_cast<const float4*>(u0 + 4 * i * NP4 + j);
+          const float v[4] = {u.x, u.y, u.z, u.w};
+#pragma unroll
+          for (int q = 0; q < 4; ++q) {
+            s[i][0] = fmaf(t[q].x, v[q], s[i][0]);
+            s[i][1] = fmaf(t[q].y, v[q], s[i][1]);
+            s[i][2] = fmaf(t[q].z, v[q], s[i][2]);
+            s[i][3] = fmaf(t[q].w, v[q], s[i][3]);
           }
         }
+      }
+      // e_i = sum of u s over this lane's outputs, then over the 8 lanes of the row
+      // group: lane og ends with row row0 + 4 og (the same tree for every row)
+      float e[8];
+      const int i0 = 32 * ob + og * 4;
 #pragma unroll
-        for (int q = 0; q < RPT; ++q)
-#pragma unroll
-          for (int ii = 0; ii < 8; ++ii)
-            if (i0 + ii < NP) e[q] = fmaf(u0[q * THREADS * RS + i0 + ii], sacc[q][ii], e[q]);
+      for (int i = 0; i < 8; ++i) {
+        const float4 u = i0 < NP4 ? *reinterpret_cast<const float4*>(u0 + 4 * i * NP4 + i0)
+                                  : make_float4(0.f, 0.f, 0.f, 0.f);
+        e[i] = fmaf(u.w, s[i][3], fmaf(u.z, s[i][2], fmaf(u.y, s[i][1], u.x * s[i][0])));
       }
 #pragma unroll
-      for (int q = 0; q < RPT; ++q)
-        if (threadIdx.x + q * THREADS < nr) acc += double(w[q]) * double(e[q]);
+      for (int h = 4; h; h >>= 1) {
+        const bool high = og & h;
+#pragma unroll
+        for (int i = 0; i < h; ++i) {
+          const float keep = high ? e[i + h] : e[i], send = high ? e[i] : e[i + h];
+          e[i] = keep + __shfl_xor_sync(0xffffffffu, send, h);
+        }
+      }
+      const int row = row0 + 4 * og;
+      if (row < nr) acc += double(sW[row]) * double(e[0]);
     }
   }
   tc::cp_async_wait_all();
-  __shared__ double sw[(THREADS + 31) / 32];
+  __shared__ double sw[S::WARPS];
 #pragma unroll
   for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
-  if ((threadIdx.x & 31) == 0) sw[threadIdx.x >> 5] = acc;
-  __syncthreads();
-  if (threadIdx.x == 0) {
-    double t = 0.0;
-    for (int w = 0; w < (THREADS + 31) / 32; ++w) t += sw[w];
-    A.partials[blockIdx.x] = t;
-  }
-}
-
-// Any order: one warp per element, lane i forms (M u_c)_i (M symmetric, read
-// column-wise = coalesced) and u_i (M u_c)_i in FP32, scaled by J_k in FP64.
-__global__ void __launch_bounds__(kEnergyThreads) energy_kernel(const EnergyArgs A) {
-  const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
-  constexpr int nw = kEnergyThreads / 32;
-  double acc = 0.0;
-  for (int k = A.k0 + blockIdx.x * nw + warp; k < A.k1; k += gridDim.x * nw) {
-    float ek = 0.f;
-    const float4 mw = A.mat ? __ldg(A.mat + size_t(k) * kMatVecs) : make_float4(1.f, 1.f, 1.f, 1.f);
-    for (int c = 0; c < 6; ++c) {
-      const float* uk = A.u + (size_t(c) * A.K + k) * A.Np;
-      const float w = c < 3 ? mw.z : mw.w;          // eps for E, mu for H (1 in vacuum)
-      for (int i = lane; i < A.Np; i += 32) {
-        float s = 0.f;
-        for (int j = 0; j < A.Np; ++j) s = fmaf(__ldg(A.M + j * A.Np + i), __ldg(uk + j), s);
-        ek = fmaf(w * __ldg(uk + i), s, ek);
-      }
-    }
-#pragma unroll
-    for (int o = 16; o; o >>= 1) ek += __shfl_xor_sync(0xffffffffu, ek, o);
-    const float J = reinterpret_cast<const float*>(A.geo)[size_t(k) * kGeoWords + 9];
-    acc += double(J) * double(ek);
-  }
-  __shared__ double sw[nw];
   if (lane == 0) sw[warp] = acc;
   __syncthreads();
-  if (threadIdx.x == 0) {
+  if (tid == 0) {
     double t = 0.0;
-    for (int w = 0; w < nw; ++w) t += sw[w];
+    for (int w = 0; w < S::WARPS; ++w) t += sw[w];
     A.partials[blockIdx.x] = t;
   }
 }
@@ -379,56 +236,119 @@ __global__ void energy_finalize(const double* partials, int n, double* result) {
   if (threadIdx.x == 0) result[0] = 0.5 * t;
 }
 
-int energy_grid(int num_sms) { return 4 * num_sms; }
-
-template <int NP>
-static cudaError_t launch_energy_rows(const EnergyArgs& a, int grid, cudaStream_t s) {
-  constexpr int bytes = EnergyRowsShape<NP>::BYTES;
-  static bool attr[16] = {};
-  int dev = 0;
-  cudaError_t err = cudaGetDevice(&dev);
-  if (err != cudaSuccess) return err;
-  if (!attr[dev & 15]) {
-    err = cudaFuncSetAttribute(energy_rows_kernel<NP>,
-                               cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
-    if (err != cudaSuccess) return err;
-    attr[dev & 15] = true;
+// Orders 1 and 2 (4 and 10 nodes): a row per thread straight from global memory, the
+// packed triangle in shared memory.  Reading the fields bounds it; staging rows for a
+// product this small cost more than it saved (a dg_energy call, staged before and now:
+// N = 1, 705 894 tets 121 -> 64 us; N = 2, 279 936 tets 83 -> 50 us).
+template <int NP, bool VEC>
+__global__ void __launch_bounds__(256) energy_row_kernel(const EnergyArgs A) {
+  constexpr int NT = NP * (NP + 1) / 2, NT4 = (NT + 3) & ~3;
+  __shared__ __align__(16) float sT[NT4];              // rows i: T_ii, T_i+1,i, ...
+  for (int x = threadIdx.x; x < NT; x += 256) {
+    int i = 0, o = x;
+    while (o >= NP - i) o -= NP - i++;
+    sT[x] = __ldg(A.T + (i + o) * 32 + i);
   }
-  energy_rows_kernel<NP><<<grid, kEnergyRows, bytes, s>>>(a);
+  __syncthreads();
+  const unsigned Kr = unsigned(A.k1 - A.k0), rows = 6u * Kr;
+  double acc = 0.0;
+#pragma unroll 2
+  for (unsigned g = blockIdx.x * 256 + threadIdx.x; g < rows; g += gridDim.x * 256) {
+    const unsigned c = g / Kr;
+    const int64_t k = A.k0 + int64_t(g - c * Kr);
+    const float* row = A.u + (int64_t(c) * A.K + k) * NP;
+    float u[NP];
+    if constexpr (VEC) {
+#pragma unroll
+      for (int q = 0; q < NP / 4; ++q) {
+        const float4 x = __ldg(reinterpret_cast<const float4*>(row) + q);
+        u[4 * q] = x.x; u[4 * q + 1] = x.y; u[4 * q + 2] = x.z; u[4 * q + 3] = x.w;
+      }
+    } else {
+#pragma unroll
+      for (int j = 0; j < NP; ++j) u[j] = __ldg(row + j);
+    }
+    float wgt = __ldg(A.J + k);
+    if (A.mat) {
+      const float4 m = __ldg(A.mat + k * kMatVecs);
+      wgt *= c < 3 ? m.z : m.w;
+    }
+    float e = 0.f;
+    int x = 0;
+#pragma unroll
+    for (int i = 0; i < NP; ++i) {
+      float s = 0.f;
+#pragma unroll
+      for (int j = i; j < NP; ++j) s = fmaf(sT[x++], u[j], s);
+      e = fmaf(u[i], s, e);
+    }
+    acc += double(wgt) * double(e);
+  }
+  __shared__ double sw[8];
+#pragma unroll
+  for (int o = 16; o; o >>= 1) acc += __shfl_xor_sync(0xffffffffu, acc, o);
+  if ((threadIdx.x & 31) == 0) sw[threadIdx.x >> 5] = acc;
+  __syncthreads();
+  if (threadIdx.x == 0) {
+    double t = 0.0;
+    for (int w = 0; w < 8; ++w) t += sw[w];
+    A.partials[blockIdx.x] = t;
+  }
+}
+
+// Partial sums kept per mesh; a launch uses as many as it has blocks.
+int energy_grid(int num_sms) { return 8 * num_sms; }
+
+template <int NP, bool VEC>
+static cudaError_t launch_energy_row(const EnergyArgs& a, int num_sms, int* grid, cudaStream_t s) {
+  const int64_t blocks = (6 * int64_t(a.k1 - a.k0) + 255) / 256;
+  *grid = int(std::min<int64_t>(blocks, energy_grid(num_sms)));
+  energy_row_kernel<NP, VEC><<<*grid, 256, 0, s>>>(a);
   return cudaGetLastError();
 }
 
-template <int NP, int THREADS, int RPT>
-static cudaError_t launch_energy_wide(const EnergyArgs& a, int grid, cudaStream_t s) {
-  constexpr int bytes = EnergyWideShape<NP, THREADS, RPT>::BYTES;
-  auto kern = energy_wide_kernel<NP, THREADS, RPT>;
-  static bool attr[16] = {};
+template <int N>
+static cudaError_t launch_energy_n(const EnergyArgs& a, int num_sms, int* grid, cudaStream_t s) {
+  using S = EnergyShape<N>;
+  // 16-byte copies where every row starts on a 16-byte boundary
+  const bool vec = S::NP % 4 == 0 && reinterpret_cast<uintptr_t>(a.u) % 16 == 0;
+  auto kern = energy_tile_kernel<N, false>;
+  if constexpr (S::NP % 4 == 0)
+    if (vec) kern = energy_tile_kernel<N, true>;
+  static int occ[2][16] = {};                          // [vec][device]: blocks per SM
   int dev = 0;
   cudaError_t err = cudaGetDevice(&dev);
   if (err != cudaSuccess) return err;
-  if (!attr[dev & 15]) {
-    err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, bytes);
+  int& o = occ[vec ? 1 : 0][dev & 15];
+  if (o == 0) {
+    err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, S::BYTES);
     if (err != cudaSuccess) return err;
-    attr[dev & 15] = true;
+    int n = 0;
+    err = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&n, kern, S::THREADS, S::BYTES);
+    if (err != cudaSuccess) return err;
+    o = n < 1 ? 1 : n > 8 ? 8 : n;
   }
-  kern<<<grid, THREADS, bytes, s>>>(a);
+  const int64_t passes = (6 * int64_t(a.k1 - a.k0) + S::ROWS - 1) / S::ROWS;
+  *grid = int(std::min<int64_t>(passes, int64_t(num_sms) * o));
+  kern<<<*grid, S::THREADS, S::BYTES, s>>>(a);
   return cudaGetLastError();
 }
 
-cudaError_t launch_energy_partials(const EnergyArgs& a, int grid, cudaStream_t s) {
-  switch (a.Np) {
-    case 4: return launch_energy_rows<4>(a, grid, s);
-    case 10: return launch_energy_rows<10>(a, grid, s);
-    case 20: return launch_energy_rows<20>(a, grid, s);
-    case 35: return launch_energy_wide<35, 256, 2>(a, grid, s);
-    case 56: return launch_energy_rows<56>(a, grid, s);
-    case 84: return launch_energy_wide<84, 256, 2>(a, grid, s);
-    case 120: return launch_energy_wide<120, 128, 2>(a, grid, s);
-    case 165: return launch_energy_wide<165, 64, 2>(a, grid, s);
-    case 220: return launch_energy_wide<220, 32, 1>(a, grid, s);
-    default:
-      energy_kernel<<<grid, kEnergyThreads, 0, s>>>(a);
-      return cudaGetLastError();
+cudaError_t launch_energy_partials(int N, const EnergyArgs& a, int num_sms, int* grid,
+                                   cudaStream_t s) {
+  switch (N) {
+    case 1: return reinterpret_cast<uintptr_t>(a.u) % 16 == 0
+                       ? launch_energy_row<4, true>(a, num_sms, grid, s)
+                       : launch_energy_row<4, false>(a, num_sms, grid, s);
+    case 2: return launch_energy_row<10, false>(a, num_sms, grid, s);
+    case 3: return launch_energy_n<3>(a, num_sms, grid, s);
+    case 4: return launch_energy_n<4>(a, num_sms, grid, s);
+    case 5: return launch_energy_n<5>(a, num_sms, grid, s);
+    case 6: return launch_energy_n<6>(a, num_sms, grid, s);
+    case 7: return launch_energy_n<7>(a, num_sms, grid, s);
+    case 8: return launch_energy_n<8>(a, num_sms, grid, s);
+    case 9: return launch_energy_n<9>(a, num_sms, grid, s);
+    default: return cudaErrorInvalidValue;
   }
 }
 
@@ -445,9 +365,11 @@ struct DeviceState {
   int Np = 0, Nfp = 0;
   int num_sms = 0;
   float4* geo = nullptr;
+  float* J = nullptr;           // Jacobians alone (energy)
   float4* D4 = nullptr;
   float4* LIFT4 = nullptr;
   float* M = nullptr;
+  float* T = nullptr;
   unsigned char* fmask = nullptr;
   unsigned char* perm = nullptr;
   float* u_work = nullptr;      // second state buffer for the stage ping-pong
@@ -573,6 +495,7 @@ struct OrderOps {
   float4* D4 = nullptr;
   float4* LIFT4 = nullptr;
   float* M = nullptr;
+  float* T = nullptr;           // weighted triangle of M, energy kernel layout
   unsigned char* fmask = nullptr;
   unsigned char* perm = nullptr;
   void* tcB = nullptr;
@@ -613,6 +536,18 @@ static int order_ops(const dg_mesh* m, int dev, OrderOps& out, std::string& err)
   if ((rc = upload(&o.LIFT4, L4, err))) return rc;
   std::vector<float> Mf(m->ops.M.begin(), m->ops.M.end());
   if ((rc = upload(&o.M, Mf, err))) return rc;
+  // T_ji = M_ii, 2 M_ij (j > i): [output block of 32][j from the block's first][output]
+  {
+    const int NP4 = (Np + 3) & ~3;
+    std::vector<float> T;
+    for (int i0 = 0; i0 < Np; i0 += 32)
+      for (int j = i0; j < NP4; ++j)
+        for (int i = i0; i < i0 + 32; ++i)
+          T.push_back(i >= Np || j >= Np || j < i
+                          ? 0.f
+                          : (j > i ? 2.f : 1.f) * static_cast<float>(m->ops.M[i * Np + j]));
+    if ((rc = upload(&o.T, T, err))) return rc;
+  }
   std::vector<unsigned char> fm(m->ops.Fmask.begin(), m->ops.Fmask.end());
   if ((rc = upload(&o.fmask, fm, err))) return rc;
   std::vector<unsigned char> pm(m->ops.perm.begin(), m->ops.perm.end());
@@ -751,6 +686,7 @@ int ensure_device(dg_mesh* m, std::string& err) {
   d->D4 = ops.D4;
   d->LIFT4 = ops.LIFT4;
   d->M = ops.M;
+  d->T = ops.T;
   d->fmask = ops.fmask;
   d->perm = ops.perm;
   d->tcB = ops.tcB;
@@ -767,9 +703,10 @@ int ensure_device(dg_mesh* m, std::string& err) {
   const size_t geo_b = static_cast<size_t>(K) * dgdev::kGeoWords * 4;
   const size_t mat_b = m->eps.empty() ? 0 : static_cast<size_t>(K) * dgdev::kMatVecs * 16;
   const size_t tcg_b = static_cast<size_t>(ntiles) * d->tc_geo_stride * 4;
-  const size_t o_mat = up(geo_b), o_tcg = o_mat + up(mat_b), o_part = o_tcg + up(tcg_b);
-  const size_t o_res = o_part + up(sizeof(double) * d->egrid), o_stat = o_res + 256;
-  const size_t total = o_stat + 256;
+  const size_t o_J = up(geo_b), o_mat = o_J + up(static_cast<size_t>(K) * 4), o_tcg = o_mat + up(mat_b), o_part = o_tcg + up(tcg_b);
+  // the energy and the status word share 16 bytes: one copy reads both
+  const size_t o_res = o_part + up(sizeof(double) * d->egrid), o_stat = o_res + 8;
+  const size_t total = o_res + 256;
   std::vector<unsigned char> host(o_part, 0);
 
   // geometry records
@@ -778,6 +715,7 @@ int ensure_device(dg_mesh* m, std::string& err) {
     float* g = &geo[k * dgdev::kGeoWords];
     for (int a = 0; a < 9; ++a) g[a] = static_cast<float>(m->metric[a * K + k]);
     g[9] = static_cast<float>(m->J[k]);
+    reinterpret_cast<float*>(host.data() + o_J)[k] = g[9];
     uint32_t codes = 0;
     for (int f = 0; f < 4; ++f) {
       const int c = m->nbr_code[4 * k + f];
@@ -833,8 +771,9 @@ int ensure_device(dg_mesh* m, std::string& err) {
   DG_CUDA(cudaMalloc(&d->arena, total), "cudaMalloc");
   unsigned char* base = static_cast<unsigned char*>(d->arena);
   DG_CUDA(cudaMemcpy(base, host.data(), host.size(), cudaMemcpyHostToDevice), "cudaMemcpy H2D");
-  DG_CUDA(cudaMemset(base + o_stat, 0, 256), "cudaMemset");
+  DG_CUDA(cudaMemset(base + o_res, 0, 256), "cudaMemset");
   d->geo = reinterpret_cast<float4*>(base);
+  d->J = reinterpret_cast<float*>(base + o_J);
   d->mat = mat_b ? reinterpret_cast<float4*>(base + o_mat) : nullptr;
   d->tcgeo = reinterpret_cast<float*>(base + o_tcg);
   d->partials = reinterpret_cast<double*>(base + o_part);
@@ -1105,16 +1044,21 @@ int device_step(dg_mesh* m, float* u, float* res, double dt, int nsteps, void* s
   return step_impl(m, u, res, dt, nsteps, static_cast<cudaStream_t>(stream), err);
 }
 
-// Reads (and clears) the pipeline status word; only after a synchronisation.
-static int check_status(dg_mesh* m, std::string& err) {
-  int st = 0;
-  DG_CUDA(cudaMemcpy(&st, m->dev->status, sizeof(int), cudaMemcpyDeviceToHost), "cudaMemcpy D2H");
+// Clears a set status word and reports it.
+static int report_status(dg_mesh* m, int st, std::string& err) {
   if (st != 0) {
     DG_CUDA(cudaMemset(m->dev->status, 0, sizeof(int)), "cudaMemset");
     err = "tensor-core stage: an MMA completion wait timed out (results invalid)";
     return DG_ERR_CUDA;
   }
   return DG_OK;
+}
+
+// Reads (and clears) the pipeline status word; only after a synchronisation.
+static int check_status(dg_mesh* m, std::string& err) {
+  int st = 0;
+  DG_CUDA(cudaMemcpy(&st, m->dev->status, sizeof(int), cudaMemcpyDeviceToHost), "cudaMemcpy D2H");
+  return report_status(m, st, err);
 }
 
 int device_wait_selftest(dg_mesh* m, uint32_t polls, double* seconds, std::string& err) {
@@ -1132,17 +1076,22 @@ int device_wait_selftest(dg_mesh* m, uint32_t polls, double* seconds, std::strin
 static int energy_impl(dg_mesh* m, const float* u, double* out, cudaStream_t s,
                        std::string& err, int64_t k0 = 0, int64_t k1 = -1) {
   DeviceState* d = m->dev;
-  dgdev::EnergyArgs a{u, d->M, d->geo, static_cast<int>(d->K), d->Np, d->partials, d->result,
+  dgdev::EnergyArgs a{u, d->T, d->J, static_cast<int>(d->K), d->Np, d->partials, d->result,
                       static_cast<int>(k0), static_cast<int>(k1 < 0 ? d->K : k1), d->mat};
-  DG_CUDA(traced(m, s, 2, [&] { return dgdev::launch_energy_partials(a, d->egrid, s); }),
+  int grid = 0;
+  DG_CUDA(traced(m, s, 2, [&] {
+            return dgdev::launch_energy_partials(m->N, a, d->num_sms, &grid, s);
+          }), "energy kernel launch");
+  DG_CUDA(traced(m, s, 3, [&] { return dgdev::launch_energy_final(a, grid, s); }),
           "energy kernel launch");
-  DG_CUDA(traced(m, s, 3, [&] { return dgdev::launch_energy_final(a, d->egrid, s); }),
-          "energy kernel launch");
-  double h = 0.0;
-  DG_CUDA(cudaMemcpyAsync(&h, d->result, sizeof(double), cudaMemcpyDeviceToHost, s),
+  // the energy and, beside it, the status word of the stages before it
+  struct { double energy; int status, unused; } r = {0.0, 0, 0};
+  static_assert(sizeof(r) == 16, "layout");
+  DG_CUDA(cudaMemcpyAsync(&r, d->result, sizeof(r), cudaMemcpyDeviceToHost, s),
           "cudaMemcpyAsync D2H");
   DG_CUDA(cudaStreamSynchronize(s), "cudaStreamSynchronize");
-  if (int rc = check_status(m, err)) return rc;
+  if (int rc = report_status(m, r.status, err)) return rc;
+  const double h = r.energy;
   *out = h;
   m->last_launches = 2;
   if (!std::isfinite(h)) { err = "energy is not finite (unstable run)"; return DG_ERR_UNSTABLE; }

@@ -139,16 +139,18 @@ cudaError_t launch_wait_selftest(int* status, uint32_t polls, unsigned long long
 
 struct EnergyArgs {
   const float* u;      // [6][K][Np]
-  const float* M;      // [Np][Np]
-  const float4* geo;   // for J
+  const float* T;      // weighted triangle of M (device.cu, energy kernel)
+  const float* J;      // [K]
   int K, Np;
-  double* partials;    // [grid]
+  double* partials;    // [blocks of the launch <= energy_grid]
   double* result;      // [1]
   int k0, k1;          // elements k0 <= k < k1 (0, K: the whole mesh)
   const float4* mat;   // material record (E rows weighted by eps, H rows by mu), or null
 };
 int energy_grid(int num_sms);
-cudaError_t launch_energy_partials(const EnergyArgs& a, int grid, cudaStream_t s);
+// *grid receives the number of blocks (partial sums) launched.
+cudaError_t launch_energy_partials(int N, const EnergyArgs& a, int num_sms, int* grid,
+                                   cudaStream_t s);
 cudaError_t launch_energy_final(const EnergyArgs& a, int grid, cudaStream_t s);
 
 }  // namespace dgdev
