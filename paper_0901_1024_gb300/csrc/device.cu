@@ -783,28 +783,32 @@ int ensure_device(dg_mesh* m, std::string& err) {
 }
 
 // The kernel family of a stage call.
-enum class Path { fp32, tc, tw, tw_shifted };
+enum class Path { fp32, direct, tc, tw, tw_shifted };
 
 // DG_STAGE_TC and orders 2..7 of DG_STAGE_AUTO: the tensor-core stages of
 // tc_stage.cuh and tc_stage_t.cuh, which move whole tiles with bulk copies and need
 // every field chunk 16-byte aligned ((K * Np) % 4 == 0 and 16-byte aligned buffers).
 // DG_STAGE_AUTO at orders 8 and 9: the streamed-operator tensor-core stage, shifted
-// where chunks are off the 16-byte grid.  Everything else: FP32 CUDA cores (N = 1,
-// Np = 4, is faster there than on the tensor cores).
+// where chunks are off the 16-byte grid.  Everything else: FP32 CUDA cores, at order 1
+// (faster there than on the tensor cores, Np = 4) one thread per element for 16-byte
+// aligned buffers and the default tile shape, else tiles.
 static Path stage_path(const dg_mesh* m, std::initializer_list<const void*> bufs) {
-  if (m->stage_impl == DG_STAGE_FP32) return Path::fp32;
   bool aligned = (m->K * m->ops.Np) % 4 == 0;
   for (const void* p : bufs) aligned = aligned && reinterpret_cast<uintptr_t>(p) % 16 == 0;
+  const Path cuda_cores = m->N == 1 && aligned && m->stage_shape == 0 ? Path::direct : Path::fp32;
+  if (m->stage_impl == DG_STAGE_FP32) return cuda_cores;
   if (m->stage_impl == DG_STAGE_AUTO) {
-    if (m->N == 1) return Path::fp32;
+    if (m->N == 1) return cuda_cores;
     if (tw_order(m->N))
       return aligned ? Path::tw : m->ops.Np % 4 != 0 ? Path::tw_shifted : Path::fp32;
   }
   return m->N <= dgdev::kTcMaxOrder && aligned ? Path::tc : Path::fp32;
 }
 
+static bool on_cuda_cores(Path p) { return p == Path::fp32 || p == Path::direct; }
+
 static int stage_tile(const dg_mesh* m, Path p) {
-  return p == Path::fp32 ? dgdev::stage_tile_elems(m->N, m->stage_shape)
+  return on_cuda_cores(p) ? dgdev::stage_tile_elems(m->N, m->stage_shape)
                          : dgdev::tc_tile_elems(m->N);
 }
 
@@ -835,6 +839,23 @@ static cudaError_t launch_path(const dg_mesh* m, Path p, bool rk, const dgdev::S
                                cudaStream_t s) {
   const int sms = m->dev->num_sms;
   switch (p) {
+    case Path::direct: {
+      dgdev::StageArgs e = a;                        // tiles -> elements
+      const int E = stage_tile(m, p);
+      e.tile0 = a.tile0 * E;
+      e.num_tiles = std::min(a.num_tiles * E, a.K - e.tile0);
+      dgdev::DirectOps<1> o;
+      for (int i = 0; i < o.Np; ++i) {
+        for (int j = 0; j < o.Np; ++j) {
+          o.D[0][i][j] = static_cast<float>(m->ops.Dr[i * o.Np + j]);
+          o.D[1][i][j] = static_cast<float>(m->ops.Ds[i * o.Np + j]);
+          o.D[2][i][j] = static_cast<float>(m->ops.Dt[i * o.Np + j]);
+        }
+        for (int f = 0; f < 4 * o.Nfp; ++f)
+          o.L[i][f] = static_cast<float>(m->ops.LIFT[i * 4 * o.Nfp + f]);
+      }
+      return dgdev::launch_direct_stage(rk, e, o, s);
+    }
     case Path::tc: return dgdev::launch_tc_stage(m->N, rk, a, sms, s);
     case Path::tw: return dgdev::launch_tw_stage(m->N, rk, false, a, sms, s);
     case Path::tw_shifted: return dgdev::launch_tw_stage(m->N, rk, true, a, sms, s);
@@ -850,7 +871,7 @@ int device_rhs(dg_mesh* m, const float* u, float* rhs, void* stream, std::string
   dgdev::StageArgs a = stage_args(m, p);
   a.u_in = u;
   a.rhs = rhs;
-  DG_CUDA(traced(m, s, p == Path::fp32 ? 1 : 5, [&] { return launch_path(m, p, false, a, s); }),
+  DG_CUDA(traced(m, s, on_cuda_cores(p) ? 1 : 5, [&] { return launch_path(m, p, false, a, s); }),
           "stage kernel launch");
   m->last_launches = 1;
   return DG_OK;
@@ -885,7 +906,7 @@ static int step_impl(dg_mesh* m, float* u, float* res, double dt, int nsteps, cu
       a.u_out = dst;
       a.a = static_cast<float>(kRkA[i]);
       a.b = static_cast<float>(kRkB[i]);
-      DG_CUDA(traced(m, s, p == Path::fp32 ? 0 : 4, [&] { return launch_path(m, p, true, a, s); }),
+      DG_CUDA(traced(m, s, on_cuda_cores(p) ? 0 : 4, [&] { return launch_path(m, p, true, a, s); }),
               "stage kernel launch");
       ++launches;
       float* nsrc = dst;
@@ -931,7 +952,7 @@ int device_stage(dg_mesh* m, const float* u_in, float* u_out, float* res, int st
   a.dt_elem = dt_elem;
   a.a = static_cast<float>(kRkA[stage]);
   a.b = static_cast<float>(kRkB[stage]);
-  DG_CUDA(traced(m, s, p == Path::fp32 ? 0 : 4, [&] { return launch_path(m, p, true, a, s); }),
+  DG_CUDA(traced(m, s, on_cuda_cores(p) ? 0 : 4, [&] { return launch_path(m, p, true, a, s); }),
           "stage kernel launch");
   m->last_launches = 1;
   return DG_OK;

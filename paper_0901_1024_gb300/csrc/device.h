@@ -137,6 +137,15 @@ cudaError_t launch_tc_stage(int N, bool rk, const StageArgs& a, int num_sms, cud
 cudaError_t launch_wait_selftest(int* status, uint32_t polls, unsigned long long* ns,
                                  cudaStream_t s);
 
+// One-thread-per-element stage (direct_stage.cuh): the operators as a kernel
+// parameter; StageArgs' tile0 and num_tiles count elements.  16-byte aligned buffers.
+template <int N> struct DirectOps {
+  static constexpr int Np = (N + 1) * (N + 2) * (N + 3) / 6, Nfp = (N + 1) * (N + 2) / 2;
+  float D[3][Np][Np];      // Dr, Ds, Dt
+  float L[Np][4 * Nfp];    // LIFT
+};
+cudaError_t launch_direct_stage(bool rk, const StageArgs& a, const DirectOps<1>& o, cudaStream_t s);
+
 struct EnergyArgs {
   const float* u;      // [6][K][Np]
   const float* T;      // weighted triangle of M (device.cu, energy kernel)
