@@ -54,31 +54,13 @@
 
 namespace dgdev {
 
-// The node nearest the centroid among the equispaced nodes (same order as the
-// Warp & Blend nodes: first coordinate fastest).
-__host__ __device__ constexpr int tw_central_node(int N) {
-  int best = 0, at = 0, n = 0;
-  for (int k = 0; k <= N; ++k)
-    for (int j = 0; j + k <= N; ++j)
-      for (int i = 0; i + j + k <= N; ++i, ++n) {
-        const int l = N - i - j - k;
-        const int d = (4 * i - N) * (4 * i - N) + (4 * j - N) * (4 * j - N) +
-                      (4 * k - N) * (4 * k - N) + (4 * l - N) * (4 * l - N);
-        if (n == 0 || d < best) {
-          best = d;
-          at = n;
-        }
-      }
-  return at;
-}
-
 template <int N> struct TwDims {
   static constexpr int Np = (N + 1) * (N + 2) * (N + 3) / 6;
   static constexpr int Nfp = (N + 1) * (N + 2) / 2;
   static constexpr int NF = 4 * Nfp;
   static constexpr int E = tc_tile_elems(N);
   static constexpr int ROWS = 6 * E;
-  static constexpr int JC = tw_central_node(N);
+  static constexpr int JC = tc_central_node(N);
   static constexpr int JB = tw_jblocks(N);             // node blocks of 16
   static constexpr int FB = tw_fblocks(N);             // face-node blocks of 16
   static constexpr int KS = 3 * JB + FB;               // K steps of a tile

@@ -1,5 +1,5 @@
-"""The streamed-operator tensor-core stage (orders 8 and 9 by default) against the
-FP64 oracle and the FP32 stage: ragged and full tiles, several tiles per CTA,
+"""The streamed-operator tensor-core stage (orders 8 and 9 by default) and the order-4
+stage for field chunks off the 16-byte grid against the FP64 oracle and the FP32 stage: ragged and full tiles, several tiles per CTA,
 field chunks off the 16-byte grid, materials and absorbing faces, per-element
 steps, element ranges, and its accuracy against the FP32 stage's."""
 from __future__ import annotations
@@ -45,10 +45,12 @@ def _rhs(torch, mesh, u32, impl):
 
 
 # K = 48 and 162 end in ragged tiles (of 20 at order 8, of 16 at order 9; 48 is whole at
-# order 9); 160 is whole at both; 161 and 159 put order 8's chunks off the 16-byte grid
+# order 9); 160 is whole at both; 161 and 159 put order 8's chunks off the 16-byte grid, K
+# not a multiple of 4 order 4's (tiles of 20; all three offsets)
 @pytest.mark.parametrize("ext", [False, True])
 @pytest.mark.parametrize("N,K", [(8, 4), (8, 48), (8, 160), (8, 161), (8, 162), (8, 159), (9, 1),
-                                 (9, 48), (9, 160), (9, 161)])
+                                 (9, 48), (9, 160), (9, 161), (4, 1), (4, 2), (4, 3), (4, 21),
+                                 (4, 22), (4, 23), (4, 161), (4, 162)])
 def test_rhs_against_the_oracle(env, N, K, ext):
     torch, dg = env
     verts, tets = kuhn_box_mesh(3, 0.15, 10 + N)
@@ -70,7 +72,7 @@ def test_rhs_against_the_oracle(env, N, K, ext):
     assert rel(got, want) < RHS_TOL
 
 
-@pytest.mark.parametrize("N,K", [(8, 3072 + 7), (8, 3072 + 8), (9, 2600)])
+@pytest.mark.parametrize("N,K", [(8, 3072 + 7), (8, 3072 + 8), (9, 2600), (4, 3041), (4, 4374 - 1)])
 def test_several_tiles_per_cta(env, N, K):
     """More tiles than SMs: the rings wrap from tile to tile."""
     torch, dg = env
@@ -90,7 +92,7 @@ def test_several_tiles_per_cta(env, N, K):
         assert rel(a, b.astype(np.float64)) < RHS_TOL * 10
 
 
-@pytest.mark.parametrize("N,K", [(8, 162), (8, 164), (9, 162)])
+@pytest.mark.parametrize("N,K", [(8, 162), (8, 164), (9, 162), (4, 162), (4, 163)])
 def test_element_steps_and_ranges(env, N, K):
     """Per-element steps equal the scalar step bit for bit where they agree, and two
     ranges of tiles equal the whole mesh."""
