@@ -67,7 +67,11 @@ __host__ __device__ constexpr int tc_central_node(int N) {
   return at;
 }
 
-template <int N, bool SH = false> struct TcDims {
+// PAIR: two CTAs of 12 warps an SM, each with half the tensor memory.  At order 2 a tile
+// is so small that its chain of barriers, not its work, takes the time; two chains share
+// the SM.
+template <int N, bool SH = false, bool PAIR = false> struct TcDims {
+  static constexpr int ORDER = N;
   static constexpr int Np = (N + 1) * (N + 2) * (N + 3) / 6;
   static constexpr int Nfp = (N + 1) * (N + 2) / 2;
   static constexpr int NF = 4 * Nfp;
@@ -80,7 +84,8 @@ template <int N, bool SH = false> struct TcDims {
   static constexpr int KSTEPS = KT / 16;
   static constexpr int ACOLS = KT / 2;                // tensor-memory columns per A piece
   static constexpr int NN = (Np + 15) & ~15;          // MMA N
-  static constexpr int BUF_COLS = 256;                // columns per pipeline buffer
+  static constexpr int TMEM = PAIR ? 256 : 512;       // tensor-memory columns of a CTA
+  static constexpr int BUF_COLS = TMEM / 2;           // columns per pipeline buffer
   static_assert(2 * ACOLS + NN <= BUF_COLS, "tensor-memory buffer overflow");
   static constexpr int COLS_G = KB / 2;               // columns of one mu block
   static constexpr int COLS_F = KF / 2;               // columns of the flux block
@@ -90,8 +95,9 @@ template <int N, bool SH = false> struct TcDims {
   static constexpr bool MIXED_SPLIT = N != 4;
   static constexpr int FSTR = NF + 2;                // flux row stride: 8-byte pair reads of
                                                       // a warp's 32 rows are conflict-free
-  static constexpr int THREADS = 640;                 // 4 epilogue + 16 producer warps
-  static constexpr int PRODUCERS = 512;
+  static constexpr int ROLES = PAIR ? 2 : 4;          // producer roles of 4 warps each
+  static constexpr int PRODUCERS = 128 * ROLES;
+  static constexpr int THREADS = 128 + PRODUCERS;     // 4 epilogue warps + the producers
   // Flux items (face nodes): the producers take elements 0 .. E0-1 in at most
   // two rounds; the face nodes of elements E0 .. E-1 are computed one tile
   // ahead by epilogue warps 1..3 (warp 0 issues the MMAs), which otherwise
@@ -117,14 +123,14 @@ template <int N, bool SH = false> struct TcDims {
   static constexpr int F2_FLOATS = 6 * (E - E0) * FSTR;      // epilogue-computed flux rows
   static constexpr int OFF_F2 = OFF_F + F_FLOATS * 4;         // [2 tiles][6][E - E0][FSTR]
   static constexpr int OFF_BND = OFF_F2 + 2 * F2_FLOATS * 4;  // [2 tiles][4 roles][128] row bounds
-  static constexpr int OFF_SC = OFF_BND + 2 * 4 * 128 * 4;   // [4][128] row scales
+  static constexpr int OFF_SC = OFF_BND + 2 * 4 * 128 * 4;   // [4][128] row scales (tiles t mod 4)
   static constexpr int OFF_TAB = OFF_SC + 4 * 128 * 4;
   static constexpr int SMEM = OFF_TAB + TAB_BYTES;
   static_assert((U_FLOATS * 4) % 16 == 0 && (E * Np * 4) % 16 == 0, "bulk-copy alignment");
   static_assert(OFF_U % 16 == 0 && OFF_R % 16 == 0 && OFF_G % 16 == 0 && OFF_F % 16 == 0 &&
                 OFF_TAB % 16 == 0, "alignment");
   static_assert((G_FLOATS * 4) % 16 == 0, "geometry block must be a 16-byte multiple");
-  static_assert(SMEM <= 226 * 1024, "shared memory budget");
+  static_assert(SMEM <= (PAIR ? 112 : 226) * 1024, "shared memory budget");
 };
 
 static_assert(tc_b_bytes(4) == 2 * TcDims<4>::B_BYTES, "B buffer size formula");
@@ -316,6 +322,13 @@ __device__ __forceinline__ void tc_store_sh(const StageArgs& A, const TcShift& s
   __syncwarp();
 }
 
+// The largest of a row's bounds, one per producer role.
+template <class D> __device__ __forceinline__ float tc_row_bound(const float* bnd, int row) {
+  float b = fmaxf(bnd[row], bnd[128 + row]);
+  if constexpr (D::ROLES == 4) b = fmaxf(b, fmaxf(bnd[256 + row], bnd[384 + row]));
+  return b;
+}
+
 // One g-block builder row (a producer thread of role 0 or 1) of tile t.
 struct GRow {
   const float* su;
@@ -336,16 +349,15 @@ struct GRow {
 // bound, splits g^mu = sign (r_mu,a U_a - r_mu,b U_b) into tensor memory.
 // REF: the fields enter less their value at a node near the centroid (D annihilates
 // constants), so that every rounding scales with the field's variation in the element.
-template <int N, int P0, int NPH, bool REF>
+template <class D, int P0, int NPH, bool REF>
 __device__ __forceinline__ void build_g_half(const GRow& g, int role) {
-  using D = TcDims<N>;
   constexpr int E = D::E, Np = D::Np;
   float2 ua[NPH], ub[NPH];
   float umax = 0.f;
   const float* pa = g.su + g.fa * g.us + g.re * Np;
   const float* pb = g.su + g.fb * g.us + g.re * Np;
-  const float ra = REF && g.live ? pa[tc_central_node(N)] : 0.f;
-  const float rb = REF && g.live ? pb[tc_central_node(N)] : 0.f;
+  const float ra = REF && g.live ? pa[tc_central_node(D::ORDER)] : 0.f;
+  const float rb = REF && g.live ? pb[tc_central_node(D::ORDER)] : 0.f;
 #pragma unroll
   for (int i = 0; i < NPH; ++i) {
     const int j = 2 * (P0 + i);
@@ -377,8 +389,7 @@ __device__ __forceinline__ void build_g_half(const GRow& g, int role) {
   float* bnd = g.sBound + (g.t & 1) * 512;
   bnd[role * 128 + g.row] = cmax * umax;
   named_sync(2, D::PRODUCERS);            // row bounds published
-  const float s = row_scale(fmaxf(fmaxf(bnd[g.row], bnd[128 + g.row]),
-                                  fmaxf(bnd[256 + g.row], bnd[384 + g.row])));
+  const float s = row_scale(tc_row_bound<D>(bnd, g.row));
   // A[buf] is free once the MMAs of tile t-2 have completed
   if (g.t >= 2) wait_or_flag(g.mma_done, ((g.t - 2) >> 1) & 1, g.status);
   tc::fence_after_sync();
@@ -414,9 +425,8 @@ struct FRow {
 // Columns [P0, P0 + NPH) of the flux block of one A row: loads those flux values
 // (8-byte pairs), publishes their maximum, and after the barrier splits them,
 // scaled by the row's power of two, into tensor memory.
-template <int N, int P0, int NPH>
+template <class D, int P0, int NPH>
 __device__ __forceinline__ void build_flux_half(const FRow& g, int role) {
-  using D = TcDims<N>;
   constexpr int NF = D::NF;
   const float2* frow = reinterpret_cast<const float2*>(g.frow);
   float2 w[NPH];
@@ -429,8 +439,7 @@ __device__ __forceinline__ void build_flux_half(const FRow& g, int role) {
   float* bnd = g.sBound + (g.t & 1) * 512;
   bnd[role * 128 + g.row] = fmax;
   named_sync(2, D::PRODUCERS);                     // row bounds published
-  const float s = row_scale(fmaxf(fmaxf(bnd[g.row], bnd[128 + g.row]),
-                                  fmaxf(bnd[256 + g.row], bnd[384 + g.row])));
+  const float s = row_scale(tc_row_bound<D>(bnd, g.row));
   // A[buf] is free once the MMAs of tile t-2 have completed
   if (g.t >= 2) wait_or_flag(g.mma_done, ((g.t - 2) >> 1) & 1, g.status);
   tc::fence_after_sync();
@@ -602,9 +611,9 @@ __device__ __forceinline__ void tc_flux_items(const uint32_t (&item)[NI], const 
 // so the truncating accumulator loses no more than it did (smooth fields, one right-hand
 // side: 1.45e-7 relative L2 error against 1.52e-7; an order-4 mesh of 82 943 tetrahedra
 // 149 us a stage against 330, of 1 295 8.4 against 29).
-template <int N, bool RK, bool EXT, bool SH = false>
+template <int N, bool RK, bool EXT, bool SH = false, bool PAIR = false>
 __device__ __forceinline__ void tc_stage_body(const StageArgs& A, const int cta, const int ncta) {
-  using D = TcDims<N, SH>;
+  using D = TcDims<N, SH, PAIR>;
   constexpr int E = D::E, Np = D::Np, Nfp = D::Nfp, FSTR = D::FSTR;
   extern __shared__ __align__(1024) unsigned char smem[];
   __shared__ uint32_t s_tmem;
@@ -632,7 +641,7 @@ __device__ __forceinline__ void tc_stage_body(const StageArgs& A, const int cta,
   // ---- set-up: B pieces (one bulk copy, constant data: it may overlap the
   // previous kernel), face-node table, tensor memory, barriers ----------------
   for (int i = tid; i < 4 * Nfp; i += D::THREADS) sFmask[i] = __ldg(A.fmask + i);
-  if (warp == 0) tc::tmem_alloc(&s_tmem, 512);
+  if (warp == 0) tc::tmem_alloc(&s_tmem, D::TMEM);
   if (tid == 0) {
     tc::mbar_init(&s_b_full, 1);
     for (int i = 0; i < D::NSU; ++i) tc::mbar_init(&s_u_full[i], SH ? 33 : 1);
@@ -857,7 +866,8 @@ __device__ __forceinline__ void tc_stage_body(const StageArgs& A, const int cta,
     // Warps 4..19 compute the fluxes of tile t together, then build its A rows:
     // per tensor-memory lane quarter, roles 0 and 1 (warps 4-7, 8-11) the first
     // and second half of the node range of the three g blocks, roles 2 and 3
-    // (warps 12-15, 16-19) the first and second half of the flux block.
+    // (warps 12-15, 16-19) the first and second half of the flux block.  PAIR: warps
+    // 4..11, role 0 the g blocks and role 1 the flux block.
     const int pt = tid - 128;
     const int role = (warp - 4) >> 2, quarter = warp & 3;
     const int row = quarter * 32 + lane;
@@ -889,13 +899,13 @@ __device__ __forceinline__ void tc_stage_body(const StageArgs& A, const int cta,
       // and go on with the g blocks.
       // (barriers 3 and 4 alternate by tile, so the epilogue threads' arrivals
       // for tile t+1 never meet tile t's)
-      if (role < 2) named_arrive(3 + (t & 1), D::FCOUNT);
+      if (role < D::ROLES / 2) named_arrive(3 + (t & 1), D::FCOUNT);
       else named_sync(3 + (t & 1), D::FCOUNT);
       // ---- A rows of tile t
       const bool live = row < D::ROWS && re < Ev;
       const uint32_t a_hi = tbase + lane_off + buf * D::BUF_COLS;
       const uint32_t a_lo = a_hi + D::ACOLS;
-      if (role >= 2) {
+      if (role >= D::ROLES / 2) {
         // roles 2 and 3: the first and second half of the flux block's columns
         constexpr int HC = (D::COLS_F + 1) / 2;
         // flux rows of elements >= E0 are in the epilogue threads' buffer
@@ -904,20 +914,24 @@ __device__ __forceinline__ void tc_stage_body(const StageArgs& A, const int cta,
                                              (rc * (E - D::E0) + re - D::E0) * FSTR;
         const FRow fr{frow, sBound, t, row, live, a_hi + 3 * D::COLS_G,
                       a_lo + 3 * D::COLS_G, &s_mma_done[buf], A.status};
-        if (role == 2)
-          build_flux_half<N, 0, HC>(fr, 2);
+        if constexpr (PAIR)
+          build_flux_half<D, 0, D::COLS_F>(fr, role);
+        else if (role == 2)
+          build_flux_half<D, 0, HC>(fr, 2);
         else
-          build_flux_half<N, HC, D::COLS_F - HC>(fr, 3);
+          build_flux_half<D, HC, D::COLS_F - HC>(fr, 3);
       } else {
         // roles 0 and 1 split the node range: node pairs [0, H) and [H, KB/2) of
         // all three g blocks, each loading only its half of the two curl fields
         constexpr int H = (D::KB / 2 + 1) / 2;
         const GRow gr{su, sg, sBound, sScale, us, t, row, rc, re, o, fa, fb, sgn, live, a_hi, a_lo,
                       &s_mma_done[buf], A.status};
-        if (role == 0)
-          build_g_half<N, 0, H, SH>(gr, 0);
+        if constexpr (PAIR)
+          build_g_half<D, 0, D::KB / 2, SH>(gr, 0);
+        else if (role == 0)
+          build_g_half<D, 0, H, SH>(gr, 0);
         else
-          build_g_half<N, H, D::KB / 2 - H, SH>(gr, 1);
+          build_g_half<D, H, D::KB / 2 - H, SH>(gr, 1);
       }
       tc::tmem_st_wait();
       tc::fence_before_sync();
@@ -927,18 +941,22 @@ __device__ __forceinline__ void tc_stage_body(const StageArgs& A, const int cta,
 
   tc::fence_before_sync();
   __syncthreads();
-  if (warp == 0) tc::tmem_dealloc(tbase, 512);
+  if (warp == 0) tc::tmem_dealloc(tbase, D::TMEM);
 }
 
+// Orders run as two CTAs an SM (when launched alone; a mixed launch has one CTA shape).
+__host__ __device__ constexpr bool tc_pair(int N) { return N == 2; }
+
 template <int N, bool RK, bool EXT, bool SH>
-__global__ void __launch_bounds__(TcDims<N>::THREADS, 1) tc_stage_kernel(const __grid_constant__ StageArgs A) {
+__global__ void __launch_bounds__(TcDims<N, SH, tc_pair(N)>::THREADS, tc_pair(N) ? 2 : 1)
+tc_stage_kernel(const __grid_constant__ StageArgs A) {
   pdl_launch_dependents();
-  tc_stage_body<N, RK, EXT, SH>(A, int(blockIdx.x), int(gridDim.x));
+  tc_stage_body<N, RK, EXT, SH, tc_pair(N)>(A, int(blockIdx.x), int(gridDim.x));
 }
 
 template <int N, bool SH>
 cudaError_t launch_tc_stage_shift(bool rk, const StageArgs& a, int num_sms, cudaStream_t s) {
-  using D = TcDims<N, SH>;
+  using D = TcDims<N, SH, tc_pair(N)>;
   static bool attr[2][2][16] = {};      // [rk][ext][device]: attribute set
   int dev = 0;
   cudaError_t err = cudaGetDevice(&dev);
@@ -948,15 +966,15 @@ cudaError_t launch_tc_stage_shift(bool rk, const StageArgs& a, int num_sms, cuda
   auto kern = rk ? (ext ? tc_stage_kernel<N, true, true, SH> : tc_stage_kernel<N, true, false, SH>)
                  : (ext ? tc_stage_kernel<N, false, true, SH> : tc_stage_kernel<N, false, false, SH>);
   // at least 120 KB of shared memory: never two CTAs (each takes all 512
-  // tensor-memory columns) on one SM
-  constexpr int smem = D::SMEM > 120 * 1024 ? D::SMEM : 120 * 1024;
+  // tensor-memory columns) on one SM; PAIR: at least 80 KB, never three
+  constexpr int least = (tc_pair(N) ? 80 : 120) * 1024, smem = D::SMEM > least ? D::SMEM : least;
   bool& done = attr[rk ? 1 : 0][ext ? 1 : 0][dev];
   if (!done) {
     err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (err != cudaSuccess) return err;
     done = true;
   }
-  const int grid = a.num_tiles < num_sms ? a.num_tiles : num_sms;
+  const int ctas = num_sms * (tc_pair(N) ? 2 : 1), grid = a.num_tiles < ctas ? a.num_tiles : ctas;
   if (grid <= 0) return cudaSuccess;
   return launch_pdl(kern, grid, D::THREADS, smem, s, a);
 }
