@@ -67,9 +67,9 @@ __host__ __device__ constexpr int tc_central_node(int N) {
   return at;
 }
 
-// PAIR: two CTAs of 12 warps an SM, each with half the tensor memory.  At order 2 a tile
-// is so small that its chain of barriers, not its work, takes the time; two chains share
-// the SM.
+// PAIR: two CTAs of 12 warps an SM, each with half the tensor memory (orders 2 and 3).
+// Their tiles are so small that the chain of barriers, not the work, takes the time (4 k
+// cycles a tile at order 2, a third of the issue slots used); two chains share the SM.
 template <int N, bool SH = false, bool PAIR = false> struct TcDims {
   static constexpr int ORDER = N;
   static constexpr int Np = (N + 1) * (N + 2) * (N + 3) / 6;
@@ -85,8 +85,14 @@ template <int N, bool SH = false, bool PAIR = false> struct TcDims {
   static constexpr int ACOLS = KT / 2;                // tensor-memory columns per A piece
   static constexpr int NN = (Np + 15) & ~15;          // MMA N
   static constexpr int TMEM = PAIR ? 256 : 512;       // tensor-memory columns of a CTA
-  static constexpr int BUF_COLS = TMEM / 2;           // columns per pipeline buffer
-  static_assert(2 * ACOLS + NN <= BUF_COLS, "tensor-memory buffer overflow");
+  // A double buffered beside the double-buffered accumulator where both fit, else single
+  static constexpr int ABUF = 2 * (2 * ACOLS + NN) <= TMEM ? 2 : 1;
+  static constexpr int BUF_COLS = TMEM / 2;           // columns per pipeline buffer (ABUF = 2)
+  static_assert(ABUF == 2 || 2 * ACOLS + 2 * NN <= TMEM, "tensor-memory buffer overflow");
+  __host__ __device__ static constexpr int a_col(int t) { return ABUF == 2 ? (t & 1) * BUF_COLS : 0; }
+  __host__ __device__ static constexpr int acc_col(int t) {
+    return ABUF == 2 ? (t & 1) * BUF_COLS + 2 * ACOLS : 2 * ACOLS + (t & 1) * NN;
+  }
   static constexpr int COLS_G = KB / 2;               // columns of one mu block
   static constexpr int COLS_F = KF / 2;               // columns of the flux block
   // FP16 split residual by mixed-precision FMAs (fewer instructions: 1-1.5 %
@@ -102,12 +108,12 @@ template <int N, bool SH = false, bool PAIR = false> struct TcDims {
   // two rounds; the face nodes of elements E0 .. E-1 are computed one tile
   // ahead by epilogue warps 1..3 (warp 0 issues the MMAs), which otherwise
   // wait for A.
-  static constexpr int E0 = 2 * PRODUCERS / NF < E ? 2 * PRODUCERS / NF : E;
+  static constexpr int E0 = PAIR || 2 * PRODUCERS / NF >= E ? E : 2 * PRODUCERS / NF;
   static constexpr int ITEMS = (E0 * NF + PRODUCERS - 1) / PRODUCERS;  // flux items per producer
   static constexpr int EPI = (E - E0) * NF;              // face nodes of the epilogue threads
   static constexpr int EITEMS = EPI ? (EPI + 95) / 96 : 1;   // per thread of warps 1..3
   static constexpr int FCOUNT = PRODUCERS + (EPI ? 128 : 0);  // threads at the flux barrier
-  static constexpr int NSU = 5, NSR = 2;              // ring slots: fields+geometry, RK register
+  static constexpr int NSU = PAIR && N == 3 ? 4 : 5, NSR = 2;              // ring slots: fields+geometry, RK register
   // shared memory (bytes)
   // one tile of one state array (shifted: field stride up to 3 values longer)
   static constexpr int U_FLOATS = 6 * (E * Np + (SH ? 4 : 0));
@@ -390,8 +396,8 @@ __device__ __forceinline__ void build_g_half(const GRow& g, int role) {
   bnd[role * 128 + g.row] = cmax * umax;
   named_sync(2, D::PRODUCERS);            // row bounds published
   const float s = row_scale(tc_row_bound<D>(bnd, g.row));
-  // A[buf] is free once the MMAs of tile t-2 have completed
-  if (g.t >= 2) wait_or_flag(g.mma_done, ((g.t - 2) >> 1) & 1, g.status);
+  // A's buffer is free once the MMAs of tile t - ABUF have completed
+  if (g.t >= D::ABUF) wait_or_flag(g.mma_done, ((g.t - D::ABUF) >> 1) & 1, g.status);
   tc::fence_after_sync();
   if (role == 0) g.sScale[(g.t & 3) * 128 + g.row] = s;
   // the scale goes on the fields, not on the metric terms: s may be as large
@@ -440,8 +446,8 @@ __device__ __forceinline__ void build_flux_half(const FRow& g, int role) {
   bnd[role * 128 + g.row] = fmax;
   named_sync(2, D::PRODUCERS);                     // row bounds published
   const float s = row_scale(tc_row_bound<D>(bnd, g.row));
-  // A[buf] is free once the MMAs of tile t-2 have completed
-  if (g.t >= 2) wait_or_flag(g.mma_done, ((g.t - 2) >> 1) & 1, g.status);
+  // A's buffer is free once the MMAs of tile t - ABUF have completed
+  if (g.t >= D::ABUF) wait_or_flag(g.mma_done, ((g.t - D::ABUF) >> 1) & 1, g.status);
   tc::fence_after_sync();
   split_store_fn<NPH, P0, D::MIXED_SPLIT>([&](int p) { return __fmul2_rn(w[p - P0], f2(s)); }, g.a_hi, g.a_lo);
 }
@@ -718,8 +724,8 @@ __device__ __forceinline__ void tc_stage_body(const StageArgs& A, const int cta,
         const int buf = j & 1;
         if (j == 0) wait_or_flag(&s_b_full, 0, A.status);   // B pieces in shared memory
         tc::fence_after_sync();
-        const uint32_t d_acc = tbase + buf * D::BUF_COLS + 2 * D::ACOLS;
-        const uint32_t a_base = tbase + buf * D::BUF_COLS;
+        const uint32_t d_acc = tbase + D::acc_col(j);
+        const uint32_t a_base = tbase + D::a_col(j);
         const uint64_t b_hi = tc::smem_desc(tc::smem_u32(smem + D::OFF_B), LBO, 128);
         const uint64_t b_lo = b_hi + uint64_t(D::B_BYTES >> 4);
 #pragma unroll
@@ -781,7 +787,7 @@ __device__ __forceinline__ void tc_stage_body(const StageArgs& A, const int cta,
         if (RK) wait_or_flag(&s_r_full[t % D::NSR], (t / D::NSR) & 1, A.status);
         tc::fence_after_sync();
         uint32_t acc[D::NN];
-        tmem_load_cols<D::NN>(tbase + lane_off + buf * D::BUF_COLS + 2 * D::ACOLS, acc);
+        tmem_load_cols<D::NN>(tbase + lane_off + D::acc_col(t), acc);
         tc::tmem_ld_wait();
         tc::fence_before_sync();
         if (row < D::ROWS && re < Ev) {
@@ -893,7 +899,16 @@ __device__ __forceinline__ void tc_stage_body(const StageArgs& A, const int cta,
       // ---- fluxes (Alg. 3) of elements 0 .. E0-1 (the epilogue warps did the
       // rest one tile ahead).  F was last read in the build of tile t-1, before
       // its barrier.
-      tc_flux_items<N, EXT, D::ITEMS>(item, A, k0, Ev, su, us, sg, F, E, 0);
+#pragma unroll
+      for (int q = 0; q < D::ITEMS; q += 2) {         // two items' operands in registers
+        if (q + 1 < D::ITEMS) {
+          const uint32_t it[2] = {item[q], item[q + 1]};
+          tc_flux_items<N, EXT, 2>(it, A, k0, Ev, su, us, sg, F, E, 0);
+        } else {
+          const uint32_t it[1] = {item[q]};
+          tc_flux_items<N, EXT, 1>(it, A, k0, Ev, su, us, sg, F, E, 0);
+        }
+      }
       // The flux buffer is complete once every producer has stored its items:
       // roles 2 and 3 (which read it) wait for that; roles 0 and 1 only signal
       // and go on with the g blocks.
@@ -903,7 +918,7 @@ __device__ __forceinline__ void tc_stage_body(const StageArgs& A, const int cta,
       else named_sync(3 + (t & 1), D::FCOUNT);
       // ---- A rows of tile t
       const bool live = row < D::ROWS && re < Ev;
-      const uint32_t a_hi = tbase + lane_off + buf * D::BUF_COLS;
+      const uint32_t a_hi = tbase + lane_off + D::a_col(t);
       const uint32_t a_lo = a_hi + D::ACOLS;
       if (role >= D::ROLES / 2) {
         // roles 2 and 3: the first and second half of the flux block's columns
@@ -913,7 +928,7 @@ __device__ __forceinline__ void tc_stage_body(const StageArgs& A, const int cta,
                                        : sF2 + (t & 1) * D::F2_FLOATS +
                                              (rc * (E - D::E0) + re - D::E0) * FSTR;
         const FRow fr{frow, sBound, t, row, live, a_hi + 3 * D::COLS_G,
-                      a_lo + 3 * D::COLS_G, &s_mma_done[buf], A.status};
+                      a_lo + 3 * D::COLS_G, &s_mma_done[(t - D::ABUF) & 1], A.status};
         if constexpr (PAIR)
           build_flux_half<D, 0, D::COLS_F>(fr, role);
         else if (role == 2)
@@ -925,7 +940,7 @@ __device__ __forceinline__ void tc_stage_body(const StageArgs& A, const int cta,
         // all three g blocks, each loading only its half of the two curl fields
         constexpr int H = (D::KB / 2 + 1) / 2;
         const GRow gr{su, sg, sBound, sScale, us, t, row, rc, re, o, fa, fb, sgn, live, a_hi, a_lo,
-                      &s_mma_done[buf], A.status};
+                      &s_mma_done[(t - D::ABUF) & 1], A.status};
         if constexpr (PAIR)
           build_g_half<D, 0, D::KB / 2, SH>(gr, 0);
         else if (role == 0)
@@ -944,37 +959,36 @@ __device__ __forceinline__ void tc_stage_body(const StageArgs& A, const int cta,
   if (warp == 0) tc::tmem_dealloc(tbase, D::TMEM);
 }
 
-// Orders run as two CTAs an SM (when launched alone; a mixed launch has one CTA shape).
-__host__ __device__ constexpr bool tc_pair(int N) { return N == 2; }
-
-template <int N, bool RK, bool EXT, bool SH>
-__global__ void __launch_bounds__(TcDims<N, SH, tc_pair(N)>::THREADS, tc_pair(N) ? 2 : 1)
+template <int N, bool RK, bool EXT, bool SH, bool PAIR>
+__global__ void __launch_bounds__(TcDims<N, SH, PAIR>::THREADS, PAIR ? 2 : 1)
 tc_stage_kernel(const __grid_constant__ StageArgs A) {
   pdl_launch_dependents();
-  tc_stage_body<N, RK, EXT, SH, tc_pair(N)>(A, int(blockIdx.x), int(gridDim.x));
+  tc_stage_body<N, RK, EXT, SH, PAIR>(A, int(blockIdx.x), int(gridDim.x));
 }
 
-template <int N, bool SH>
-cudaError_t launch_tc_stage_shift(bool rk, const StageArgs& a, int num_sms, cudaStream_t s) {
-  using D = TcDims<N, SH, tc_pair(N)>;
+template <int N, bool SH, bool PAIR>
+cudaError_t launch_tc_stage_form(bool rk, const StageArgs& a, int num_sms, cudaStream_t s) {
+  using D = TcDims<N, SH, PAIR>;
   static bool attr[2][2][16] = {};      // [rk][ext][device]: attribute set
   int dev = 0;
   cudaError_t err = cudaGetDevice(&dev);
   if (err != cudaSuccess) return err;
   dev &= 15;
   const bool ext = a.mat || a.absorbing;
-  auto kern = rk ? (ext ? tc_stage_kernel<N, true, true, SH> : tc_stage_kernel<N, true, false, SH>)
-                 : (ext ? tc_stage_kernel<N, false, true, SH> : tc_stage_kernel<N, false, false, SH>);
+  auto kern = rk ? (ext ? tc_stage_kernel<N, true, true, SH, PAIR>
+                        : tc_stage_kernel<N, true, false, SH, PAIR>)
+                 : (ext ? tc_stage_kernel<N, false, true, SH, PAIR>
+                        : tc_stage_kernel<N, false, false, SH, PAIR>);
   // at least 120 KB of shared memory: never two CTAs (each takes all 512
   // tensor-memory columns) on one SM; PAIR: at least 80 KB, never three
-  constexpr int least = (tc_pair(N) ? 80 : 120) * 1024, smem = D::SMEM > least ? D::SMEM : least;
+  constexpr int least = (PAIR ? 80 : 120) * 1024, smem = D::SMEM > least ? D::SMEM : least;
   bool& done = attr[rk ? 1 : 0][ext ? 1 : 0][dev];
   if (!done) {
     err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
     if (err != cudaSuccess) return err;
     done = true;
   }
-  const int ctas = num_sms * (tc_pair(N) ? 2 : 1), grid = a.num_tiles < ctas ? a.num_tiles : ctas;
+  const int ctas = num_sms * (PAIR ? 2 : 1), grid = a.num_tiles < ctas ? a.num_tiles : ctas;
   if (grid <= 0) return cudaSuccess;
   return launch_pdl(kern, grid, D::THREADS, smem, s, a);
 }
@@ -985,8 +999,18 @@ cudaError_t launch_tc_stage_shift(bool rk, const StageArgs& a, int num_sms, cuda
 template <int N>
 cudaError_t launch_tc_stage_n(bool rk, bool shifted, const StageArgs& a, int num_sms,
                               cudaStream_t s) {
-  if (!shifted) return launch_tc_stage_shift<N, false>(rk, a, num_sms, s);
-  if constexpr (N == 4) return launch_tc_stage_shift<N, true>(rk, a, num_sms, s);
+  // Two CTAs an SM (launched alone; a mixed launch has one CTA shape): order 2 always (384
+  // tetrahedra 5.1 -> 4.8 us a stage, 279 936 176 -> 120 us), order 3 when an SM gets more
+  // than one tile (146 334 tetrahedra 130 -> 117 us, 3 072 8.7 -> 8.1 us, but 384, one tile
+  // a CTA, 6.1 -> 6.5 us).  Order 1 on request and order 4 (whose tiles do not fit twice)
+  // as one.
+  if (!shifted) {
+    if constexpr (N == 2) return launch_tc_stage_form<N, false, true>(rk, a, num_sms, s);
+    if constexpr (N == 3)
+      if (a.num_tiles > num_sms) return launch_tc_stage_form<N, false, true>(rk, a, num_sms, s);
+    if constexpr (N != 2) return launch_tc_stage_form<N, false, false>(rk, a, num_sms, s);
+  }
+  if constexpr (N == 4) return launch_tc_stage_form<N, true, false>(rk, a, num_sms, s);
   return cudaErrorInvalidValue;
 }
 
