@@ -171,12 +171,9 @@ int dg_set_boundary(dg_mesh* mesh, const int8_t* kind);
 /*
  * Implementation of the RK-stage operator (the paper notes that each operator
  * part may need its own strategy on the GPU, Section 4):
- *   DG_STAGE_AUTO   the faster kernel of each order on GB300 (default): tensor
- *                   cores as DG_STAGE_TC for N = 2..7 (at N = 4 also for K*Np
- *                   off a multiple of 4), FP32 CUDA cores for N = 1, and for N = 8, 9 a tensor-core stage with the
- *                   operator streamed through shared memory and partial sums
- *                   collected in FP32 (errors at or below DG_STAGE_FP32's; any K,
- *                   at N = 9 with 16-byte aligned field buffers);
+ *   DG_STAGE_AUTO   tensor cores for N = 2..7 (at N = 4 also for K*Np off a
+ *                   multiple of 4), FP32 CUDA cores for N = 1 and above 7
+ *                   (the faster kernel of each order on GB300; default);
  *   DG_STAGE_FP32   FP32 CUDA cores for every order;
  *   DG_STAGE_TC     tensor cores (tcgen05): the volume and lifting contractions
  *                   as one GEMM per tile with three FP16 products

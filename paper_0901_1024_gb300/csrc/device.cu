@@ -28,9 +28,6 @@ cudaError_t launch_tc_stage_n(bool rk, bool shifted, const StageArgs& a, int num
                               cudaStream_t s);
 template <int N>
 cudaError_t launch_tt_stage_n(bool rk, const StageArgs& a, int num_sms, cudaStream_t s);
-template <int N>
-cudaError_t launch_tw_stage_n(bool rk, bool shifted, const StageArgs& a, int num_sms,
-                              cudaStream_t s);
 
 // shifted: K * Np not a multiple of 4 (order 4), buffers 16-byte aligned.
 static cudaError_t launch_tc_stage(int N, bool rk, bool shifted, const StageArgs& a, int num_sms,
@@ -43,17 +40,6 @@ static cudaError_t launch_tc_stage(int N, bool rk, bool shifted, const StageArgs
     case 5: return launch_tt_stage_n<5>(rk, a, num_sms, s);
     case 6: return launch_tt_stage_n<6>(rk, a, num_sms, s);
     case 7: return launch_tt_stage_n<7>(rk, a, num_sms, s);
-    default: return cudaErrorInvalidValue;
-  }
-}
-
-// shifted: field chunks off the 16-byte grid (K * Np not a multiple of 4, or an
-// unaligned buffer).
-static cudaError_t launch_tw_stage(int N, bool rk, bool shifted, const StageArgs& a, int num_sms,
-                                   cudaStream_t s) {
-  switch (N) {
-    case 8: return launch_tw_stage_n<8>(rk, shifted, a, num_sms, s);
-    case 9: return launch_tw_stage_n<9>(rk, shifted, a, num_sms, s);
     default: return cudaErrorInvalidValue;
   }
 }
@@ -383,8 +369,8 @@ struct DeviceState {
   double* partials = nullptr;   // energy partials, one per block
   double* result = nullptr;
   int egrid = 0;
+  void* wide = nullptr;         // packed operator chunks (orders 8, 9)
   void* tcB = nullptr;          // tensor-core B pieces (orders <= kTcMaxOrder)
-  void* twB = nullptr;          // operator stream (orders of tw_order)
   float4* mat = nullptr;        // material records (meshes with materials), in the arena
   bool absorbing = false;       // some boundary face is absorbing
   float* tcgeo = nullptr;       // word-major geometry for the tensor-core stage
@@ -507,12 +493,9 @@ struct OrderOps {
   unsigned char* fmask = nullptr;
   unsigned char* perm = nullptr;
   void* tcB = nullptr;
-  void* twB = nullptr;
+  void* wide = nullptr;
   float tc_inv_bscale = 1.f;
 };
-
-// Orders that may run the streamed-operator stage (tw_stage.cuh).
-static bool tw_order(int N) { return N >= 8; }
 
 static std::mutex g_ops_mutex;
 static std::map<std::pair<int, int>, OrderOps> g_ops;
@@ -629,40 +612,27 @@ static int order_ops(const dg_mesh* m, int dev, OrderOps& out, std::string& err)
       }
     if ((rc = upload(reinterpret_cast<__half**>(&o.tcB), P, err))) return rc;
   }
-  if (tw_order(m->N)) {
-    // The streamed operator: step st of 16 K columns is node block st / 3 of
-    // Dr, Ds or Dt (st % 3), after those face-node block st - 3 JB of LIFT; zero
-    // padded, scaled by 2^p, hi then lo, [2 chunks of 8 columns][NN nodes].
-    const int N = m->N, NN = dgdev::tw_nn(N), JB = dgdev::tw_jblocks(N), KS = dgdev::tw_steps(N);
-    auto value = [&](int n, int st, int kk) -> double {
-      if (n >= Np) return 0.0;
-      if (st < 3 * JB) {
-        const int j = 16 * (st / 3) + kk, mu = st % 3;
-        const std::vector<double>& Dm = mu == 0 ? m->ops.Dr : mu == 1 ? m->ops.Ds : m->ops.Dt;
-        return j < Np ? Dm[n * Np + j] : 0.0;
-      }
-      const int f = 16 * (st - 3 * JB) + kk;
-      return f < NF ? m->ops.LIFT[n * NF + f] : 0.0;
-    };
-    double mx = 0.0;
-    for (int n = 0; n < Np; ++n)
-      for (int st = 0; st < KS; ++st)
-        for (int kk = 0; kk < 16; ++kk) mx = std::max(mx, std::fabs(value(n, st, kk)));
-    const double sB = std::ldexp(1.0, static_cast<int>(std::floor(std::log2(16384.0 / mx))));
-    o.tc_inv_bscale = static_cast<float>(1.0 / sB);
-    std::vector<__half> P(static_cast<size_t>(dgdev::tw_b_bytes(N)) / 2);
-    for (int st = 0; st < KS; ++st)
-      for (int n = 0; n < NN; ++n)
-        for (int kk = 0; kk < 16; ++kk) {
-          // the low piece from the FP64 operator: its FP32 rounding is not split too
-          const double x = value(n, st, kk) * sB;
-          const __half hi = __float2half_rn(static_cast<float>(x));
-          const __half lo = __double2half(x - static_cast<double>(__half2float(hi)));
-          const size_t off = ((static_cast<size_t>(st) * 4 + kk / 8) * NN + n) * 8 + kk % 8;
-          P[off] = hi;
-          P[off + static_cast<size_t>(2) * NN * 8] = lo;
+  if (m->N >= 8) {
+    // the register-tiled FP32 stage's operator, chunk by chunk (device.h)
+    const int JC = dgdev::wide_jc(m->N), NCH = dgdev::wide_chunks(m->N), MC = dgdev::wide_mc(m->N);
+    const int slot = dgdev::wide_chunk_bytes(m->N) / 4, NLC = NF / 4 / MC;
+    std::vector<float> W(static_cast<size_t>(NCH + NLC) * slot, 0.f);
+    for (int c = 0; c < NCH; ++c)
+      for (int i = 0; i < Np; ++i)
+        for (int jj = 0; jj < JC && c * JC + jj < Np; ++jj) {
+          const float4 d = D4[i * Np + c * JC + jj];
+          float* w = &W[static_cast<size_t>(c) * slot + (i * JC + jj) * 3];
+          w[0] = d.x;
+          w[1] = d.y;
+          w[2] = d.z;
         }
-    if ((rc = upload(reinterpret_cast<__half**>(&o.twB), P, err))) return rc;
+    for (int c = 0; c < NLC; ++c)
+      for (int i = 0; i < Np; ++i)
+        std::memcpy(&W[static_cast<size_t>(NCH + c) * slot + i * MC * 4], &L4[i * (NF / 4) + c * MC],
+                    sizeof(float4) * MC);
+    float* dw = nullptr;
+    if ((rc = upload(&dw, W, err))) return rc;
+    o.wide = dw;
   }
   g_ops[{dev, m->N}] = o;
   out = o;
@@ -698,20 +668,22 @@ int ensure_device(dg_mesh* m, std::string& err) {
   d->fmask = ops.fmask;
   d->perm = ops.perm;
   d->tcB = ops.tcB;
-  d->twB = ops.twB;
+  d->wide = ops.wide;
   d->tc_inv_bscale = ops.tc_inv_bscale;
   const int64_t K = m->K;
   const int Nfp = d->Nfp, NF = 4 * Nfp;
+  const bool tc = d->N <= dgdev::kTcMaxOrder;
   const int E = dgdev::tc_tile_elems(d->N);
   const int64_t ntiles = (K + E - 1) / E;
-  d->tc_geo_stride = dgdev::tc_geo_floats(d->N);
+  d->tc_geo_stride = tc ? dgdev::tc_geo_floats(d->N) : 0;
   d->egrid = dgdev::energy_grid(d->num_sms);
   // arena layout (bytes, each part 256-byte aligned)
   auto up = [](size_t x) { return (x + 255) & ~size_t(255); };
   const size_t geo_b = static_cast<size_t>(K) * dgdev::kGeoWords * 4;
   const size_t mat_b = m->eps.empty() ? 0 : static_cast<size_t>(K) * dgdev::kMatVecs * 16;
-  const size_t tcg_b = static_cast<size_t>(ntiles) * d->tc_geo_stride * 4;
-  const size_t o_J = up(geo_b), o_mat = o_J + up(static_cast<size_t>(K) * 4), o_tcg = o_mat + up(mat_b), o_part = o_tcg + up(tcg_b);
+  const size_t tcg_b = tc ? static_cast<size_t>(ntiles) * d->tc_geo_stride * 4 : 0;
+  const size_t o_mat = up(geo_b), o_tcg = o_mat + up(mat_b), o_J = o_tcg + up(tcg_b);
+  const size_t o_part = o_J + up(static_cast<size_t>(K) * 4);
   // the energy and the status word share 16 bytes: one copy reads both
   const size_t o_res = o_part + up(sizeof(double) * d->egrid), o_stat = o_res + 8;
   const size_t total = o_res + 256;
@@ -755,7 +727,7 @@ int ensure_device(dg_mesh* m, std::string& err) {
       }
     }
   }
-  {
+  if (tc) {
     // tiled geometry, one contiguous block per tile: word-major [kTcGeoWords][E]
     // (record words {0..8 metric, 10 codes, 12..27 faces, 28..31 neighbours} ->
     // words {0..8, 9, 10..25, 26..29}), then one byte per face node (e, m):
@@ -783,7 +755,7 @@ int ensure_device(dg_mesh* m, std::string& err) {
   d->geo = reinterpret_cast<float4*>(base);
   d->J = reinterpret_cast<float*>(base + o_J);
   d->mat = mat_b ? reinterpret_cast<float4*>(base + o_mat) : nullptr;
-  d->tcgeo = reinterpret_cast<float*>(base + o_tcg);
+  d->tcgeo = tc ? reinterpret_cast<float*>(base + o_tcg) : nullptr;
   d->partials = reinterpret_cast<double*>(base + o_part);
   d->result = reinterpret_cast<double*>(base + o_res);
   d->status = reinterpret_cast<int*>(base + o_stat);
@@ -791,16 +763,15 @@ int ensure_device(dg_mesh* m, std::string& err) {
 }
 
 // The kernel family of a stage call.
-enum class Path { fp32, direct, tc, tc_shifted, tw, tw_shifted };
+enum class Path { fp32, direct, tc, tc_shifted };
 
 // DG_STAGE_TC and orders 2..7 of DG_STAGE_AUTO: the tensor-core stages of
 // tc_stage.cuh and tc_stage_t.cuh, which move whole tiles with bulk copies and need
 // every field chunk 16-byte aligned ((K * Np) % 4 == 0 and 16-byte aligned buffers).
 // DG_STAGE_AUTO also has a form for K * Np off that grid at order 4 (82 943 tetrahedra:
-// 149 us against 330 us on CUDA cores), and at orders 8 and 9 the streamed-operator tensor-core stage, at
-// order 8 for any alignment.  Everything else: FP32 CUDA cores, at order 1 (faster there
-// than on the tensor cores, Np = 4) one thread per element for 16-byte aligned buffers
-// and the default tile shape, else tiles.
+// 149 us against 330 us on CUDA cores).  Everything else: FP32 CUDA cores, at order 1
+// (faster there than on the tensor cores, Np = 4) one thread per element for 16-byte
+// aligned buffers and the default tile shape, else tiles.
 static Path stage_path(const dg_mesh* m, std::initializer_list<const void*> bufs) {
   const bool whole = (m->K * m->ops.Np) % 4 == 0;
   bool buffers = true;
@@ -810,8 +781,6 @@ static Path stage_path(const dg_mesh* m, std::initializer_list<const void*> bufs
   if (m->stage_impl == DG_STAGE_FP32) return cuda_cores;
   if (m->stage_impl == DG_STAGE_AUTO) {
     if (m->N == 1) return cuda_cores;
-    if (m->N >= 8)
-      return aligned ? Path::tw : m->ops.Np % 4 != 0 ? Path::tw_shifted : Path::fp32;
     if (m->N == 4 && !whole && buffers) return Path::tc_shifted;
   }
   return m->N <= dgdev::kTcMaxOrder && aligned ? Path::tc : Path::fp32;
@@ -828,7 +797,7 @@ static dgdev::StageArgs stage_args(dg_mesh* m, Path p) {
   DeviceState* d = m->dev;
   dgdev::StageArgs a{};
   a.tcB = d->tcB;
-  a.twB = d->twB;
+  a.wide = d->wide;
   a.tcgeo = d->tcgeo;
   a.tc_geo_stride = d->tc_geo_stride;
   a.tc_inv_bscale = d->tc_inv_bscale;
@@ -870,8 +839,6 @@ static cudaError_t launch_path(const dg_mesh* m, Path p, bool rk, const dgdev::S
     }
     case Path::tc: return dgdev::launch_tc_stage(m->N, rk, false, a, sms, s);
     case Path::tc_shifted: return dgdev::launch_tc_stage(m->N, rk, true, a, sms, s);
-    case Path::tw: return dgdev::launch_tw_stage(m->N, rk, false, a, sms, s);
-    case Path::tw_shifted: return dgdev::launch_tw_stage(m->N, rk, true, a, sms, s);
     default: return dgdev::launch_stage(m->N, rk, a, sms, s, m->stage_shape);
   }
 }

@@ -40,6 +40,20 @@ __host__ __device__ constexpr int stage_tile_elems(int N, int shape = 0) {
                     : (N == 1 ? 8 : N <= 5 ? 16 : N == 6 ? 6 : N == 7 ? 8 : 4);
 }
 
+// Register-tiled FP32 stage (orders 8, 9): the packed operator's chunks, first Dr, Ds, Dt
+// as [row][column][r, s, t] for wide_jc columns a chunk (zero padded past the last
+// column), then LIFT as float4 [row][wide_mc], each in a slot of wide_chunk_bytes.
+__host__ __device__ constexpr int wide_jc(int N) { return N == 8 ? 14 : 20; }
+__host__ __device__ constexpr int wide_chunks(int N) {
+  return ((N + 1) * (N + 2) * (N + 3) / 6 + wide_jc(N) - 1) / wide_jc(N);
+}
+__host__ __device__ constexpr int wide_mc(int N) { return N == 8 ? 9 : 11; }
+__host__ __device__ constexpr int wide_chunk_bytes(int N) {
+  const int Np = (N + 1) * (N + 2) * (N + 3) / 6;
+  const int d = Np * wide_jc(N) * 12, l = Np * wide_mc(N) * 16;
+  return ((d > l ? d : l) + 127) / 128 * 128;
+}
+
 struct StageArgs {
   const float* u_in;       // [6][K][Np]
   float* u_out;            // [6][K][Np] (RK mode)
@@ -62,21 +76,17 @@ struct StageArgs {
   const void* tcB;          // FP16 [Dr Ds Dt LIFT] hi/lo pieces: orders <= 4 in the canonical
                             // K-major shared-memory layout, orders 5..7 as tensor-memory rows
   float tc_inv_bscale;      // 1 / (power-of-two scale applied to [Dr Ds Dt LIFT])
-  const void* twB;          // streamed-operator stage: FP16 pieces in step order (tw_stage.cuh)
+  const void* wide;         // register-tiled FP32 stage: packed operator chunks
   int* status;              // set to 1 if an MMA completion wait timed out
   int absorbing;            // 1 if any boundary face is absorbing (code kAbsorbingCode)
 };
 
 // Tensor-core stage: elements per tile.  Orders <= 4: 6 * 20 = 120 of the 128
 // MMA rows (fields are the A operand); orders 5..7: 6 * 8 = 48 MMA columns
-// (fields are the B operand, the operator sits in tensor memory); orders 8, 9
-// (fields are the A operand, the operator is streamed): 20 again, 16 at order 9
-// (the fields and fluxes of 20 would leave no room for the operator's slots).
+// (fields are the B operand, the operator sits in tensor memory).
 constexpr int kTcTileElems = 20;
 constexpr int kTtTileElems = 8;
-__host__ __device__ constexpr int tc_tile_elems(int N) {
-  return N <= 4 || N == 8 ? kTcTileElems : N == 9 ? 16 : kTtTileElems;
-}
+__host__ __device__ constexpr int tc_tile_elems(int N) { return N <= 4 ? kTcTileElems : kTtTileElems; }
 // Word-major geometry for the tensor-core stage: words 0..8 metric, 9 packed
 // neighbour codes, 10 + 4f .. 13 + 4f normal and Fscale of face f, 26 + f
 // neighbour element of face f.
@@ -97,15 +107,6 @@ __host__ __device__ constexpr int tc_b_bytes(int N) {
   return 2 * 2 * ((((N + 1) * (N + 2) * (N + 3) / 6) + 15) & ~15) *
          ((3 * ((((N + 1) * (N + 2) * (N + 3) / 6) + 1) & ~1) + 4 * ((N + 1) * (N + 2) / 2) + 15) & ~15);
 }
-
-// Streamed-operator stage (tw_stage.cuh): blocks of 16 nodes and of 16 face
-// nodes, MMA columns (nodes, padded), and bytes of the operator stream: per step
-// of 16 K columns, hi then lo, each [2 chunks of 8 columns][tw_nn nodes] FP16.
-__host__ __device__ constexpr int tw_nn(int N) { return (((N + 1) * (N + 2) * (N + 3) / 6) + 15) & ~15; }
-__host__ __device__ constexpr int tw_jblocks(int N) { return tw_nn(N) / 16; }
-__host__ __device__ constexpr int tw_fblocks(int N) { return (4 * ((N + 1) * (N + 2) / 2) + 15) / 16; }
-__host__ __device__ constexpr int tw_steps(int N) { return 3 * tw_jblocks(N) + tw_fblocks(N); }
-__host__ __device__ constexpr int tw_b_bytes(int N) { return tw_steps(N) * tw_nn(N) * 64; }
 
 // One launch over the packs of several meshes (a group per mesh): the grid's
 // CTAs are split among the groups, CTAs [first, first + count) running group g

@@ -1,3 +1,4 @@
-// Stage kernel instantiation for order N=9.
+// Stage kernel instantiations for order N=9: register tiled, and tiles of shape 1.
 #include "stage_kernel.cuh"
+#include "stage_wide.cuh"
 DG_INSTANTIATE_STAGE(9)

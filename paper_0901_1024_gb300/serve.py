@@ -282,14 +282,15 @@ class Server:
     def _choose_impl(self, N, solves):
         """(stage implementation, FP32 tile shape) of a pack: without autotuning
         the server's `impl` and the default shape; with it, the fastest of the
-        tensor-core stage (above order 7 the default one) and the FP32 stage in each tile shape,
+        tensor-core stage (orders <= 7) and the FP32 stage in each tile shape,
         timed on a scratch pack once per (device, order, decade of K)."""
         if not self.autotune:
             return self.impl, 0
         key = self._tune_key(N, solves)
         if key not in self._tuned:
             cands = [(Mesh.STAGE_FP32, 0), (Mesh.STAGE_FP32, 1)]
-            cands.insert(0, (Mesh.STAGE_TC if N <= 7 else Mesh.STAGE_AUTO, 0))
+            if N <= 7:
+                cands.insert(0, (Mesh.STAGE_TC, 0))
             times = {c: self._time_impl(N, solves, *c) for c in cands}
             self._tuned[key] = min(times, key=times.get)
         return self._tuned[key]
