@@ -11,7 +11,7 @@
 // runs of tc_tile_elems elements are nearly coalesced too.
 // Arithmetic as in stage_kernel.cuh: differentiate, chain rule and curl, flux, lifting.
 // 128 registers a thread, 16 warps an SM; the latency of the first loads bounds it.
-// 705 894 tetrahedra: 88 us a stage (62 % of the HBM roofline) against 196 us for the
+// 705 894 tetrahedra: 83 us a stage (62 % of the HBM roofline) against 196 us for the
 // tiles; without the L2 prefetch of the RK register 98 us; blocks capped at 96 or 80
 // registers 100-103 us, 64-thread blocks 97 us.
 #pragma once
@@ -81,25 +81,31 @@ direct_stage_kernel(const __grid_constant__ StageArgs A, const __grid_constant__
   }
   float rhs[6][Np];
   // local differentiation and curl, H fields first (dE/dt = curl H), then E
+  const float rx = met[0], ry = met[1], rz = met[2];
+  const float sx = met[3], sy = met[4], sz = met[5];
+  const float tx = met[6], ty = met[7], tz = met[8];
 #pragma unroll
   for (int pass = 0; pass < 2; ++pass) {
     const int fb = pass == 0 ? 3 : 0;
 #pragma unroll
     for (int i = 0; i < Np; ++i) {
-      float d[3][3];                               // [field][r, s, t]
+      float acc[3][3];                             // [field][r, s, t]
 #pragma unroll
       for (int c = 0; c < 3; ++c)
 #pragma unroll
         for (int m = 0; m < 3; ++m) {
-          float s = O.D[m][i][0] * u[fb + c][0];   // same order as the tiled stage
+          acc[c][m] = 0.f;
 #pragma unroll
-          for (int j = 1; j < Np; ++j) s = fmaf(O.D[m][i][j], u[fb + c][j], s);
-          d[c][m] = s;
+          for (int j = 0; j < Np; ++j) acc[c][m] = fmaf(O.D[m][i][j], u[fb + c][j], acc[c][m]);
         }
-      auto dx = [&](int c, int a) {                // d(field c) / dx_a
-        return fmaf(met[6 + a], d[c][2], fmaf(met[3 + a], d[c][1], met[a] * d[c][0]));
-      };
-      const float cx = dx(2, 1) - dx(1, 2), cy = dx(0, 2) - dx(2, 0), cz = dx(1, 0) - dx(0, 1);
+      float dx[3], dy[3], dz[3];
+#pragma unroll
+      for (int c = 0; c < 3; ++c) {
+        dx[c] = rx * acc[c][0] + sx * acc[c][1] + tx * acc[c][2];
+        dy[c] = ry * acc[c][0] + sy * acc[c][1] + ty * acc[c][2];
+        dz[c] = rz * acc[c][0] + sz * acc[c][1] + tz * acc[c][2];
+      }
+      const float cx = dy[2] - dz[1], cy = dz[0] - dx[2], cz = dx[1] - dy[0];
       if (pass == 0) {
         rhs[0][i] = cx; rhs[1][i] = cy; rhs[2][i] = cz;
       } else {
@@ -120,13 +126,8 @@ direct_stage_kernel(const __grid_constant__ StageArgs A, const __grid_constant__
     }
     const float nx = __ldg(g + (10 + 4 * f) * TE), ny = __ldg(g + (11 + 4 * f) * TE);
     const float nz = __ldg(g + (12 + 4 * f) * TE), sc = 0.5f * __ldg(g + (13 + 4 * f) * TE);
-    float zp = 1.f, yp = 1.f, scE = sc, scH = sc;
-    if (EXT && A.mat) {
-      const float4 cf = __ldg(A.mat + size_t(k) * kMatVecs + 1 + f);
-      zp = cf.x; yp = cf.z;
-      scE = 2.f * sc * cf.y;
-      scH = 2.f * sc * cf.w;
-    }
+    float4 cf = make_float4(1.f, 0.5f, 1.f, 0.5f);
+    if (EXT && A.mat) cf = __ldg(A.mat + size_t(k) * kMatVecs + 1 + f);
     const float al = A.alpha;
 #pragma unroll
     for (int j = 0; j < Nfp; ++j) {
@@ -154,24 +155,34 @@ direct_stage_kernel(const __grid_constant__ StageArgs A, const __grid_constant__
       const float ndE = nx * dEx + ny * dEy + nz * dEz;
       const float ndH = nx * dHx + ny * dHy + nz * dHz;
       // E: -n x dH + alpha (n (n.dE) - dE);  H: n x dE + alpha (n (n.dH) - dH), with
-      // impedances as in stage_kernel.cuh
-      float fl[6] = {-(ny * dHz - nz * dHy), -(nz * dHx - nx * dHz), -(nx * dHy - ny * dHx),
-                     (ny * dEz - nz * dEy), (nz * dEx - nx * dEz), (nx * dEy - ny * dEx)};
-      if (EXT) {
+      // impedances as in stage_kernel.cuh (the same expressions: the same rounding)
+      float fl[6];
+      if (!EXT || !A.mat) {
+        const float v[6] = {
+            -(ny * dHz - nz * dHy) + al * (nx * ndE - dEx),
+            -(nz * dHx - nx * dHz) + al * (ny * ndE - dEy),
+            -(nx * dHy - ny * dHx) + al * (nz * ndE - dEz),
+            (ny * dEz - nz * dEy) + al * (nx * ndH - dHx),
+            (nz * dEx - nx * dEz) + al * (ny * ndH - dHy),
+            (nx * dEy - ny * dEx) + al * (nz * ndH - dHz)};
 #pragma unroll
-        for (int c = 0; c < 6; ++c) fl[c] *= c < 3 ? zp : yp;
+        for (int c = 0; c < 6; ++c) fl[c] = sc * v[c];
+      } else {
+        const float fs = 2.f * sc, sE = fs * cf.y, sH = fs * cf.w;
+        const float v[6] = {
+            fmaf(al, nx * ndE - dEx, cf.x * -(ny * dHz - nz * dHy)),
+            fmaf(al, ny * ndE - dEy, cf.x * -(nz * dHx - nx * dHz)),
+            fmaf(al, nz * ndE - dEz, cf.x * -(nx * dHy - ny * dHx)),
+            fmaf(al, nx * ndH - dHx, cf.z * (ny * dEz - nz * dEy)),
+            fmaf(al, ny * ndH - dHy, cf.z * (nz * dEx - nx * dEz)),
+            fmaf(al, nz * ndH - dHz, cf.z * (nx * dEy - ny * dEx))};
+#pragma unroll
+        for (int c = 0; c < 6; ++c) fl[c] = (c < 3 ? sE : sH) * v[c];
       }
-      fl[0] += al * (nx * ndE - dEx);
-      fl[1] += al * (ny * ndE - dEy);
-      fl[2] += al * (nz * ndE - dEz);
-      fl[3] += al * (nx * ndH - dHx);
-      fl[4] += al * (ny * ndH - dHy);
-      fl[5] += al * (nz * ndH - dHz);
 #pragma unroll
       for (int c = 0; c < 6; ++c) {
-        const float x = (c < 3 ? scE : scH) * fl[c];
 #pragma unroll
-        for (int i = 0; i < Np; ++i) rhs[c][i] = fmaf(O.L[i][m], x, rhs[c][i]);
+        for (int i = 0; i < Np; ++i) rhs[c][i] = fmaf(O.L[i][m], fl[c], rhs[c][i]);
       }
     }
   }
