@@ -801,7 +801,9 @@ __device__ __forceinline__ void tc_stage_body(const StageArgs& A, const int cta,
           float* pu = su + rc * us + re * Np;
           // u and res share one shared array, so every batch is loaded before any
           // of its stores (the compiler cannot move loads across them)
-          constexpr int CH = 12;
+          // (batches of 8 at order 4: 99.6 us a stage on 82 944 tetrahedra, of 12 101.2, of 18
+          // 100.9)
+          constexpr int CH = N == 4 ? 8 : 12;
 #pragma unroll
           for (int i0 = 0; i0 < Np; i0 += CH) {
             float rv[CH], uv[CH];
