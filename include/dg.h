@@ -171,9 +171,8 @@ int dg_set_boundary(dg_mesh* mesh, const int8_t* kind);
 /*
  * Implementation of the RK-stage operator (the paper notes that each operator
  * part may need its own strategy on the GPU, Section 4):
- *   DG_STAGE_AUTO   tensor cores for N = 2..7 (at N = 4 also for K*Np off a
- *                   multiple of 4), FP32 CUDA cores for N = 1 and above 7
- *                   (the faster kernel of each order on GB300; default);
+ *   DG_STAGE_AUTO   tensor cores for N = 2..7, FP32 CUDA cores for N = 1 and
+ *                   above 7 (the faster kernel of each order on GB300; default);
  *   DG_STAGE_FP32   FP32 CUDA cores for every order;
  *   DG_STAGE_TC     tensor cores (tcgen05): the volume and lifting contractions
  *                   as one GEMM per tile with three FP16 products

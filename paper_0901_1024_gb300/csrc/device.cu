@@ -24,19 +24,16 @@ template <int N>
 cudaError_t launch_stage_n(bool rk, const StageArgs& a, int num_sms, cudaStream_t s, int shape);
 
 template <int N>
-cudaError_t launch_tc_stage_n(bool rk, bool shifted, const StageArgs& a, int num_sms,
-                              cudaStream_t s);
+cudaError_t launch_tc_stage_n(bool rk, const StageArgs& a, int num_sms, cudaStream_t s);
 template <int N>
 cudaError_t launch_tt_stage_n(bool rk, const StageArgs& a, int num_sms, cudaStream_t s);
 
-// shifted: K * Np not a multiple of 4 (order 4), buffers 16-byte aligned.
-static cudaError_t launch_tc_stage(int N, bool rk, bool shifted, const StageArgs& a, int num_sms,
-                                   cudaStream_t s) {
+cudaError_t launch_tc_stage(int N, bool rk, const StageArgs& a, int num_sms, cudaStream_t s) {
   switch (N) {
-    case 1: return launch_tc_stage_n<1>(rk, shifted, a, num_sms, s);
-    case 2: return launch_tc_stage_n<2>(rk, shifted, a, num_sms, s);
-    case 3: return launch_tc_stage_n<3>(rk, shifted, a, num_sms, s);
-    case 4: return launch_tc_stage_n<4>(rk, shifted, a, num_sms, s);
+    case 1: return launch_tc_stage_n<1>(rk, a, num_sms, s);
+    case 2: return launch_tc_stage_n<2>(rk, a, num_sms, s);
+    case 3: return launch_tc_stage_n<3>(rk, a, num_sms, s);
+    case 4: return launch_tc_stage_n<4>(rk, a, num_sms, s);
     case 5: return launch_tt_stage_n<5>(rk, a, num_sms, s);
     case 6: return launch_tt_stage_n<6>(rk, a, num_sms, s);
     case 7: return launch_tt_stage_n<7>(rk, a, num_sms, s);
@@ -763,26 +760,20 @@ int ensure_device(dg_mesh* m, std::string& err) {
 }
 
 // The kernel family of a stage call.
-enum class Path { fp32, direct, tc, tc_shifted };
+enum class Path { fp32, direct, tc };
 
 // DG_STAGE_TC and orders 2..7 of DG_STAGE_AUTO: the tensor-core stages of
 // tc_stage.cuh and tc_stage_t.cuh, which move whole tiles with bulk copies and need
 // every field chunk 16-byte aligned ((K * Np) % 4 == 0 and 16-byte aligned buffers).
-// DG_STAGE_AUTO also has a form for K * Np off that grid at order 4 (82 943 tetrahedra:
-// 149 us against 330 us on CUDA cores).  Everything else: FP32 CUDA cores, at order 1
-// (faster there than on the tensor cores, Np = 4) one thread per element for 16-byte
-// aligned buffers and the default tile shape, else tiles.
+// Everything else: FP32 CUDA cores, at order 1 (faster there than on the tensor cores,
+// Np = 4) one thread per element for 16-byte aligned buffers and the default tile shape,
+// else tiles.
 static Path stage_path(const dg_mesh* m, std::initializer_list<const void*> bufs) {
-  const bool whole = (m->K * m->ops.Np) % 4 == 0;
-  bool buffers = true;
-  for (const void* p : bufs) buffers = buffers && reinterpret_cast<uintptr_t>(p) % 16 == 0;
-  const bool aligned = whole && buffers;
+  bool aligned = (m->K * m->ops.Np) % 4 == 0;
+  for (const void* p : bufs) aligned = aligned && reinterpret_cast<uintptr_t>(p) % 16 == 0;
   const Path cuda_cores = m->N == 1 && aligned && m->stage_shape == 0 ? Path::direct : Path::fp32;
-  if (m->stage_impl == DG_STAGE_FP32) return cuda_cores;
-  if (m->stage_impl == DG_STAGE_AUTO) {
-    if (m->N == 1) return cuda_cores;
-    if (m->N == 4 && !whole && buffers) return Path::tc_shifted;
-  }
+  if (m->stage_impl == DG_STAGE_FP32 || (m->stage_impl == DG_STAGE_AUTO && m->N == 1))
+    return cuda_cores;
   return m->N <= dgdev::kTcMaxOrder && aligned ? Path::tc : Path::fp32;
 }
 
@@ -837,8 +828,7 @@ static cudaError_t launch_path(const dg_mesh* m, Path p, bool rk, const dgdev::S
       }
       return dgdev::launch_direct_stage(rk, e, o, s);
     }
-    case Path::tc: return dgdev::launch_tc_stage(m->N, rk, false, a, sms, s);
-    case Path::tc_shifted: return dgdev::launch_tc_stage(m->N, rk, true, a, sms, s);
+    case Path::tc: return dgdev::launch_tc_stage(m->N, rk, a, sms, s);
     default: return dgdev::launch_stage(m->N, rk, a, sms, s, m->stage_shape);
   }
 }

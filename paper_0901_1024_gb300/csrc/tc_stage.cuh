@@ -49,28 +49,10 @@
 
 namespace dgdev {
 
-// The node nearest the centroid among the equispaced nodes (same order as the
-// Warp & Blend nodes: first coordinate fastest).
-__host__ __device__ constexpr int tc_central_node(int N) {
-  int best = 0, at = 0, n = 0;
-  for (int k = 0; k <= N; ++k)
-    for (int j = 0; j + k <= N; ++j)
-      for (int i = 0; i + j + k <= N; ++i, ++n) {
-        const int l = N - i - j - k;
-        const int d = (4 * i - N) * (4 * i - N) + (4 * j - N) * (4 * j - N) +
-                      (4 * k - N) * (4 * k - N) + (4 * l - N) * (4 * l - N);
-        if (n == 0 || d < best) {
-          best = d;
-          at = n;
-        }
-      }
-  return at;
-}
-
 // PAIR: two CTAs of 12 warps an SM, each with half the tensor memory (orders 2 and 3).
 // Their tiles are so small that the chain of barriers, not the work, takes the time (4 k
 // cycles a tile at order 2, a third of the issue slots used); two chains share the SM.
-template <int N, bool SH = false, bool PAIR = false> struct TcDims {
+template <int N, bool PAIR = false> struct TcDims {
   static constexpr int ORDER = N;
   static constexpr int Np = (N + 1) * (N + 2) * (N + 3) / 6;
   static constexpr int Nfp = (N + 1) * (N + 2) / 2;
@@ -115,8 +97,7 @@ template <int N, bool SH = false, bool PAIR = false> struct TcDims {
   static constexpr int FCOUNT = PRODUCERS + (EPI ? 128 : 0);  // threads at the flux barrier
   static constexpr int NSU = PAIR && N == 3 ? 4 : 5, NSR = 2;              // ring slots: fields+geometry, RK register
   // shared memory (bytes)
-  // one tile of one state array (shifted: field stride up to 3 values longer)
-  static constexpr int U_FLOATS = 6 * (E * Np + (SH ? 4 : 0));
+  static constexpr int U_FLOATS = 6 * E * Np;         // one tile of one state array
   static constexpr int G_FLOATS = tc_geo_floats(N);  // word-major [w][E], node bytes
   static constexpr int F_FLOATS = ROWS * FSTR;
   static constexpr int B_BYTES = NN * KT * 2;         // one FP16 piece
@@ -250,84 +231,6 @@ __device__ __forceinline__ void tc_load_res(const StageArgs& A, int tile, float*
     tc::bulk_g2s(sr + c * D::E * D::Np, A.res + (size_t(c) * K + k0) * D::Np, fb, bar);
 }
 
-// Shifted fields (K * Np not a multiple of 4: orders 2 and 4).  A tile's fields then
-// start up to 3 values past a 16-byte boundary, field c by (c K Np) mod 4; with a field
-// stride of E * Np + (K * Np) mod 4 in shared memory every field keeps its offset, so
-// its 16-byte aligned part moves by a bulk copy and at most three values at either end
-// one by one.
-template <int N> __device__ __forceinline__ int tc_stride_sh(int K) {
-  return TcDims<N>::E * TcDims<N>::Np + ((K * TcDims<N>::Np) & 3);
-}
-// A lane's part of every such copy of n values a field (worked out once for whole
-// tiles): the loose ends it moves -- lane l the ends l and l + 32 of 36, three before and
-// three after each field's aligned part -- as offsets in shared and global memory, and
-// the bytes of the aligned parts.
-struct TcShift {
-  int us, n, so[2];                   // field stride, values a field, shared offset (-1: none)
-  uint32_t bytes;
-  size_t go[2];
-  __device__ __forceinline__ int head(int c) const { return (4 - (c * us & 3)) & 3; }
-};
-template <int N> __device__ __forceinline__ TcShift tc_shift(int K, int n) {
-  TcShift s;
-  s.us = tc_stride_sh<N>(K);
-  s.n = n;
-  s.bytes = 0;
-  for (int c = 0; c < 6; ++c) s.bytes += uint32_t((n - s.head(c)) & ~3) * 4;
-#pragma unroll
-  for (int q = 0; q < 2; ++q) {
-    const int l = (threadIdx.x & 31) + 32 * q, c = l % 18 / 3, j = l % 3;
-    const int head = s.head(c), i = l < 18 ? j : head + ((n - head) & ~3) + j;
-    const bool any = l < 36 && (l < 18 ? j < head : i < n);
-    s.so[q] = any ? c * s.us + i : -1;
-    s.go[q] = size_t(c) * K * TcDims<N>::Np + i;
-  }
-  return s;
-}
-// Whole warp: asynchronous copies of one array's tile (and the geometry block, if any)
-// into shared memory; completes *bar (count 33: the elected lane's expect_tx, every
-// lane's loose ends).
-template <int N>
-__device__ __forceinline__ void tc_load_sh(const StageArgs& A, const TcShift& s, const float* src,
-                                           int tile, float* dst, float* sg, uint64_t* bar) {
-  using D = TcDims<N, true>;
-  const size_t field = size_t(A.K) * D::Np;
-  src += size_t(tile) * (D::E * D::Np);
-  if (tc::elect_one()) {
-    tc::mbar_expect_tx(bar, s.bytes + (sg ? D::G_FLOATS * 4 : 0));
-    const float* p = src;
-#pragma unroll
-    for (int c = 0; c < 6; ++c, p += field)
-      tc::bulk_g2s(dst + c * s.us + s.head(c), p + s.head(c),
-                   uint32_t((s.n - s.head(c)) & ~3) * 4, bar);
-    if (sg) tc::bulk_g2s(sg, A.tcgeo + size_t(tile) * A.tc_geo_stride, D::G_FLOATS * 4, bar);
-  }
-  __syncwarp();
-#pragma unroll
-  for (int q = 0; q < 2; ++q)
-    if (s.so[q] >= 0) tc::cp_async4(dst + s.so[q], src + s.go[q]);
-  tc::cp_async_mbar_arrive(bar);
-}
-// Whole warp: one array's tile from shared to global memory; the bulk copies join the
-// elected lane's current bulk group.
-template <int N>
-__device__ __forceinline__ void tc_store_sh(const StageArgs& A, const TcShift& s, float* dst,
-                                            int tile, const float* src) {
-  using D = TcDims<N, true>;
-  dst += size_t(tile) * (D::E * D::Np);
-#pragma unroll
-  for (int q = 0; q < 2; ++q)
-    if (s.so[q] >= 0) dst[s.go[q]] = src[s.so[q]];
-  if (tc::elect_one()) {
-    float* p = dst;
-#pragma unroll
-    for (int c = 0; c < 6; ++c, p += size_t(A.K) * D::Np)
-      tc::bulk_s2g(p + s.head(c), src + c * s.us + s.head(c),
-                   uint32_t((s.n - s.head(c)) & ~3) * 4);
-  }
-  __syncwarp();
-}
-
 // The largest of a row's bounds, one per producer role.
 template <class D> __device__ __forceinline__ float tc_row_bound(const float* bnd, int row) {
   float b = fmaxf(bnd[row], bnd[128 + row]);
@@ -353,17 +256,13 @@ struct GRow {
 // Node pairs [P0, P0 + NPH) of the three g^mu blocks of one A row: loads that
 // part of the two curl fields, publishes its bound on |g| and, after the flux
 // bound, splits g^mu = sign (r_mu,a U_a - r_mu,b U_b) into tensor memory.
-// REF: the fields enter less their value at a node near the centroid (D annihilates
-// constants), so that every rounding scales with the field's variation in the element.
-template <class D, int P0, int NPH, bool REF>
+template <class D, int P0, int NPH>
 __device__ __forceinline__ void build_g_half(const GRow& g, int role) {
   constexpr int E = D::E, Np = D::Np;
   float2 ua[NPH], ub[NPH];
   float umax = 0.f;
   const float* pa = g.su + g.fa * g.us + g.re * Np;
   const float* pb = g.su + g.fb * g.us + g.re * Np;
-  const float ra = REF && g.live ? pa[tc_central_node(D::ORDER)] : 0.f;
-  const float rb = REF && g.live ? pb[tc_central_node(D::ORDER)] : 0.f;
 #pragma unroll
   for (int i = 0; i < NPH; ++i) {
     const int j = 2 * (P0 + i);
@@ -371,14 +270,6 @@ __device__ __forceinline__ void build_g_half(const GRow& g, int role) {
     ub[i].x = g.live ? pb[j] : 0.f;
     ua[i].y = g.live && j + 1 < Np ? pa[j + 1] : 0.f;
     ub[i].y = g.live && j + 1 < Np ? pb[j + 1] : 0.f;
-    if constexpr (REF) {
-      ua[i].x -= ra;
-      ub[i].x -= rb;
-      if (j + 1 < Np) {
-        ua[i].y -= ra;
-        ub[i].y -= rb;
-      }
-    }
     umax = fmaxf(umax, fmaxf(fmaxf(fabsf(ua[i].x), fabsf(ua[i].y)),
                              fmaxf(fabsf(ub[i].x), fabsf(ub[i].y))));
   }
@@ -612,14 +503,9 @@ __device__ __forceinline__ void tc_flux_items(const uint32_t (&item)[NI], const 
 // The stage as run by one CTA: `cta` of `ncta` CTAs that share the tiles of A
 // (tile tile0 + cta, tile0 + cta + ncta, ...).  The kernels below run it as CTA cta of
 // the grid; the mixed-order kernel runs it for the group its CTA belongs to.
-// SH: shifted fields (above), entering less a reference value and with the small
-// products (lo.lo among them) added first: the FP32 stage ran these meshes before, and
-// so the truncating accumulator loses no more than it did (smooth fields, one right-hand
-// side: 1.45e-7 relative L2 error against 1.52e-7; an order-4 mesh of 82 943 tetrahedra
-// 149 us a stage against 330, of 1 295 8.4 against 29).
-template <int N, bool RK, bool EXT, bool SH = false, bool PAIR = false>
+template <int N, bool RK, bool EXT, bool PAIR = false>
 __device__ __forceinline__ void tc_stage_body(const StageArgs& A, const int cta, const int ncta) {
-  using D = TcDims<N, SH, PAIR>;
+  using D = TcDims<N, PAIR>;
   constexpr int E = D::E, Np = D::Np, Nfp = D::Nfp, FSTR = D::FSTR;
   extern __shared__ __align__(1024) unsigned char smem[];
   __shared__ uint32_t s_tmem;
@@ -630,7 +516,7 @@ __device__ __forceinline__ void tc_stage_body(const StageArgs& A, const int cta,
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int K = A.K;
-  const int us = SH ? tc_stride_sh<N>(K) : E * Np;   // field stride in shared memory
+  constexpr int us = E * Np;                       // field stride in shared memory
   const int ntiles = (A.num_tiles - cta + ncta - 1) / ncta;
   const int base = A.tile0 + cta;                  // this CTA's first tile of the mesh
   if (ntiles <= 0) return;
@@ -650,8 +536,8 @@ __device__ __forceinline__ void tc_stage_body(const StageArgs& A, const int cta,
   if (warp == 0) tc::tmem_alloc(&s_tmem, D::TMEM);
   if (tid == 0) {
     tc::mbar_init(&s_b_full, 1);
-    for (int i = 0; i < D::NSU; ++i) tc::mbar_init(&s_u_full[i], SH ? 33 : 1);
-    for (int i = 0; i < D::NSR; ++i) tc::mbar_init(&s_r_full[i], SH ? 33 : 1);
+    for (int i = 0; i < D::NSU; ++i) tc::mbar_init(&s_u_full[i], 1);
+    for (int i = 0; i < D::NSR; ++i) tc::mbar_init(&s_r_full[i], 1);
     for (int i = 0; i < 2; ++i) {
       tc::mbar_init(&s_a_full[i], D::PRODUCERS);  // every producer thread stores A columns
       tc::mbar_init(&s_mma_done[i], 1);
@@ -672,18 +558,7 @@ __device__ __forceinline__ void tc_stage_body(const StageArgs& A, const int cta,
     const int row = warp * 32 + lane;
     const int rc = row / E, re = row - (row / E) * E;
     const uint32_t lane_off = uint32_t(warp * 32) << 16;
-    TcShift whole{};
-    if (SH && warp == 0) whole = tc_shift<N>(K, E * Np);
-    auto shift = [&](int tile) {                     // of a tile; the mesh's last may be ragged
-      return (tile + 1) * E <= K ? whole : tc_shift<N>(K, (K - tile * E) * Np);
-    };
-    if (SH && warp == 0) {
-      for (int t = 0; t < D::NSU - 1 && t < ntiles; ++t)
-        tc_load_sh<N>(A, shift(base + t * ncta), A.u_in, base + t * ncta, sU + t * D::U_FLOATS,
-                      sG + t * D::G_FLOATS, &s_u_full[t]);
-      if (RK) tc_load_sh<N>(A, shift(base), A.res, base, sR, nullptr, &s_r_full[0]);
-    }
-    if (!SH && warp == 0 && tc::elect_one()) {   // first loads: fields of tiles 0..NSU-2, res of tile 0
+    if (warp == 0 && tc::elect_one()) {   // first loads: fields of tiles 0..NSU-2, res of tile 0
       for (int t = 0; t < D::NSU - 1 && t < ntiles; ++t)
         tc_load_u<N>(A, base + t * ncta, sU + t * D::U_FLOATS, sG + t * D::G_FLOATS,
                      &s_u_full[t]);
@@ -729,10 +604,10 @@ __device__ __forceinline__ void tc_stage_body(const StageArgs& A, const int cta,
         const uint64_t b_hi = tc::smem_desc(tc::smem_u32(smem + D::OFF_B), LBO, 128);
         const uint64_t b_lo = b_hi + uint64_t(D::B_BYTES >> 4);
 #pragma unroll
-        for (int i = 0; i < (SH ? 4 : 3) * D::KSTEPS; ++i) {
-          // passes: hi.hi, hi.lo, lo.hi; SH: lo.lo, lo.hi, hi.lo, hi.hi
+        for (int i = 0; i < 3 * D::KSTEPS; ++i) {
+          // passes: hi.hi, hi.lo, lo.hi
           const int q = i / D::KSTEPS, ks = i - q * D::KSTEPS;
-          const bool al = SH ? q < 2 : q == 2, bl = SH ? q % 2 == 0 : q == 1;
+          const bool al = q == 2, bl = q == 1;
           const uint64_t bd = (bl ? b_lo : b_hi) + uint64_t((ks * 2 * LBO) >> 4);
           const uint32_t ad = a_base + (al ? D::ACOLS : 0) + ks * 8;
           tc::mma_f16_ts_warp(d_acc, ad, bd, IDESC, i > 0 ? 1u : 0u);
@@ -749,25 +624,7 @@ __device__ __forceinline__ void tc_stage_body(const StageArgs& A, const int cta,
         const int k0 = tile * E, Ev = min(E, K - k0);
         float* su = sU + (t % D::NSU) * D::U_FLOATS;
         float* sr = sR + (t % D::NSR) * D::U_FLOATS;
-        if (SH && warp == 0) {
-          if (tc::elect_one()) {
-            asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
-            tc::fence_proxy_async_smem();
-          }
-          __syncwarp();
-          if (t + D::NSU - 1 < ntiles) {
-            const int s = (t + D::NSU - 1) % D::NSU;
-            tc_load_sh<N>(A, shift(tile + (D::NSU - 1) * ncta), A.u_in,
-                          tile + (D::NSU - 1) * ncta, sU + s * D::U_FLOATS,
-                          sG + s * D::G_FLOATS, &s_u_full[s]);
-          }
-          if (RK && t + 1 < ntiles) {
-            const int s = (t + 1) % D::NSR;
-            tc_load_sh<N>(A, shift(tile + ncta), A.res, tile + ncta, sR + s * D::U_FLOATS, nullptr,
-                          &s_r_full[s]);
-          }
-        }
-        if (!SH && warp == 0 && tc::elect_one()) {
+        if (warp == 0 && tc::elect_one()) {
           // the slots of tile t-1 (its stores were issued one round ago) take
           // tiles t+NSU-1 and t+1 now, before this tile's update
           asm volatile("cp.async.bulk.wait_group.read 0;" ::: "memory");
@@ -841,17 +698,7 @@ __device__ __forceinline__ void tc_stage_body(const StageArgs& A, const int cta,
         }
         tc::fence_proxy_async_smem();
         named_sync(1, 128);
-        if (SH && warp == 0) {
-          const TcShift h = shift(tile);
-          if (RK) {
-            tc_store_sh<N>(A, h, A.u_out, tile, su);
-            tc_store_sh<N>(A, h, A.res, tile, sr);
-          } else {
-            tc_store_sh<N>(A, h, A.rhs, tile, sr);
-          }
-          if (tc::elect_one()) tc::bulk_commit();
-        }
-        if (!SH && warp == 0 && tc::elect_one()) {
+        if (warp == 0 && tc::elect_one()) {
           const uint32_t fb = uint32_t(Ev) * Np * 4;
           for (int c = 0; c < 6; ++c) {
             const size_t g = (size_t(c) * K + k0) * Np;
@@ -944,11 +791,11 @@ __device__ __forceinline__ void tc_stage_body(const StageArgs& A, const int cta,
         const GRow gr{su, sg, sBound, sScale, us, t, row, rc, re, o, fa, fb, sgn, live, a_hi, a_lo,
                       &s_mma_done[(t - D::ABUF) & 1], A.status};
         if constexpr (PAIR)
-          build_g_half<D, 0, D::KB / 2, SH>(gr, 0);
+          build_g_half<D, 0, D::KB / 2>(gr, 0);
         else if (role == 0)
-          build_g_half<D, 0, H, SH>(gr, 0);
+          build_g_half<D, 0, H>(gr, 0);
         else
-          build_g_half<D, H, D::KB / 2 - H, SH>(gr, 1);
+          build_g_half<D, H, D::KB / 2 - H>(gr, 1);
       }
       tc::tmem_st_wait();
       tc::fence_before_sync();
@@ -961,26 +808,26 @@ __device__ __forceinline__ void tc_stage_body(const StageArgs& A, const int cta,
   if (warp == 0) tc::tmem_dealloc(tbase, D::TMEM);
 }
 
-template <int N, bool RK, bool EXT, bool SH, bool PAIR>
-__global__ void __launch_bounds__(TcDims<N, SH, PAIR>::THREADS, PAIR ? 2 : 1)
+template <int N, bool RK, bool EXT, bool PAIR>
+__global__ void __launch_bounds__(TcDims<N, PAIR>::THREADS, PAIR ? 2 : 1)
 tc_stage_kernel(const __grid_constant__ StageArgs A) {
   pdl_launch_dependents();
-  tc_stage_body<N, RK, EXT, SH, PAIR>(A, int(blockIdx.x), int(gridDim.x));
+  tc_stage_body<N, RK, EXT, PAIR>(A, int(blockIdx.x), int(gridDim.x));
 }
 
-template <int N, bool SH, bool PAIR>
+template <int N, bool PAIR>
 cudaError_t launch_tc_stage_form(bool rk, const StageArgs& a, int num_sms, cudaStream_t s) {
-  using D = TcDims<N, SH, PAIR>;
+  using D = TcDims<N, PAIR>;
   static bool attr[2][2][16] = {};      // [rk][ext][device]: attribute set
   int dev = 0;
   cudaError_t err = cudaGetDevice(&dev);
   if (err != cudaSuccess) return err;
   dev &= 15;
   const bool ext = a.mat || a.absorbing;
-  auto kern = rk ? (ext ? tc_stage_kernel<N, true, true, SH, PAIR>
-                        : tc_stage_kernel<N, true, false, SH, PAIR>)
-                 : (ext ? tc_stage_kernel<N, false, true, SH, PAIR>
-                        : tc_stage_kernel<N, false, false, SH, PAIR>);
+  auto kern = rk ? (ext ? tc_stage_kernel<N, true, true, PAIR>
+                        : tc_stage_kernel<N, true, false, PAIR>)
+                 : (ext ? tc_stage_kernel<N, false, true, PAIR>
+                        : tc_stage_kernel<N, false, false, PAIR>);
   // at least 120 KB of shared memory: never two CTAs (each takes all 512
   // tensor-memory columns) on one SM; PAIR: at least 80 KB, never three
   constexpr int least = (PAIR ? 80 : 120) * 1024, smem = D::SMEM > least ? D::SMEM : least;
@@ -995,30 +842,22 @@ cudaError_t launch_tc_stage_form(bool rk, const StageArgs& a, int num_sms, cudaS
   return launch_pdl(kern, grid, D::THREADS, smem, s, a);
 }
 
-// shifted: K * Np not a multiple of 4.  Order 4 only: at order 2 (the other with Np not a
-// multiple of 4) a tile's 36 loose ends cost more than its arithmetic, and the FP32 stage
-// is as fast.
 template <int N>
-cudaError_t launch_tc_stage_n(bool rk, bool shifted, const StageArgs& a, int num_sms,
-                              cudaStream_t s) {
+cudaError_t launch_tc_stage_n(bool rk, const StageArgs& a, int num_sms, cudaStream_t s) {
   // Two CTAs an SM (launched alone; a mixed launch has one CTA shape): order 2 always (384
   // tetrahedra 5.1 -> 4.8 us a stage, 279 936 176 -> 120 us), order 3 when an SM gets more
   // than one tile (146 334 tetrahedra 130 -> 117 us, 3 072 8.7 -> 8.1 us, but 384, one tile
   // a CTA, 6.1 -> 6.5 us).  Order 1 on request and order 4 (whose tiles do not fit twice)
   // as one.
-  if (!shifted) {
-    if constexpr (N == 2) return launch_tc_stage_form<N, false, true>(rk, a, num_sms, s);
-    if constexpr (N == 3)
-      if (a.num_tiles > num_sms) return launch_tc_stage_form<N, false, true>(rk, a, num_sms, s);
-    if constexpr (N != 2) return launch_tc_stage_form<N, false, false>(rk, a, num_sms, s);
-  }
-  if constexpr (N == 4) return launch_tc_stage_form<N, true, false>(rk, a, num_sms, s);
-  return cudaErrorInvalidValue;
+  if constexpr (N == 2) return launch_tc_stage_form<N, true>(rk, a, num_sms, s);
+  if constexpr (N == 3)
+    if (a.num_tiles > num_sms) return launch_tc_stage_form<N, true>(rk, a, num_sms, s);
+  if constexpr (N != 2) return launch_tc_stage_form<N, false>(rk, a, num_sms, s);
 }
 
 }  // namespace dgdev
 
 #define DG_INSTANTIATE_TC_STAGE(NN)                                                        \
   namespace dgdev {                                                                         \
-  template cudaError_t launch_tc_stage_n<NN>(bool, bool, const StageArgs&, int, cudaStream_t);   \
+  template cudaError_t launch_tc_stage_n<NN>(bool, const StageArgs&, int, cudaStream_t);   \
   }

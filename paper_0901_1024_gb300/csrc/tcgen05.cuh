@@ -207,12 +207,6 @@ __device__ __forceinline__ void cp_async_commit() {
 __device__ __forceinline__ void cp_async_wait_all() {
   asm volatile("cp.async.wait_all;" ::: "memory");
 }
-// Arrives on the mbarrier (one of its counted arrivals) once this thread's earlier
-// cp.async copies have completed.
-__device__ __forceinline__ void cp_async_mbar_arrive(uint64_t* mbar) {
-  asm volatile("cp.async.mbarrier.arrive.noinc.shared::cta.b64 [%0];" :: "r"(smem_u32(mbar))
-               : "memory");
-}
 // Wait until at most N of this thread's committed groups are still pending.
 template <int N>
 __device__ __forceinline__ void cp_async_wait_group() {
