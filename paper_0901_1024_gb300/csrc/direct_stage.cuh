@@ -11,7 +11,7 @@
 // runs of tc_tile_elems elements are nearly coalesced too.
 // Arithmetic as in stage_kernel.cuh: differentiate, chain rule and curl, flux, lifting.
 // 128 registers a thread, 16 warps an SM; the latency of the first loads bounds it.
-// 705 894 tetrahedra: 83 us a stage (62 % of the HBM roofline) against 196 us for the
+// 705 894 tetrahedra: 83-86 us a stage (64 % of the HBM roofline) against 196 us for the
 // tiles; without the L2 prefetch of the RK register 98 us; blocks capped at 96 or 80
 // registers 100-103 us, 64-thread blocks 97 us.
 #pragma once

@@ -11,8 +11,8 @@
 //   * the operator comes packed ([chunk of JC columns][row][column][r, s, t]) through two
 //     shared-memory buffers, one bulk copy a chunk, the next chunk's under way while one
 //     is multiplied; LIFT follows through the same buffers.
-// Measured (~1.7e7 unknowns, before and after): N = 8 1014 -> 718 us, N = 9 1214 -> 937 us;
-// 38 and 41 % of the FP32 peak, the loop held up by register-bank conflicts (dispatch
+// Measured (~1.7e7 unknowns, before and after): N = 8 1014 -> 720-730 us, N = 9 1214 -> 940-950
+// us; 37 and 40 % of the FP32 peak, the loop held up by register-bank conflicts (dispatch
 // stalls).  Two CTAs an SM with half the tile 732 / 965 us, packed FP32x2 multiply-adds
 // with 8 rows a thread 747 / 957 us.
 #pragma once
