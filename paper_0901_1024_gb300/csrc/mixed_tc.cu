@@ -13,11 +13,9 @@ namespace dgdev {
 
 namespace {
 
-template <int N> constexpr int tc_smem() {
-  return TcDims<N>::SMEM > 120 * 1024 ? TcDims<N>::SMEM : 120 * 1024;
-}
 constexpr int cmax(int a, int b) { return a > b ? a : b; }
-constexpr int kMixedTcSmem = cmax(cmax(tc_smem<1>(), tc_smem<2>()), cmax(tc_smem<3>(), tc_smem<4>()));
+constexpr int kMixedTcSmem = tc_smem(512, cmax(cmax(TcDims<1>::SMEM, TcDims<2>::SMEM),
+                                               cmax(TcDims<3>::SMEM, TcDims<4>::SMEM)));
 static_assert(TcDims<1>::THREADS == 640 && TcDims<4>::THREADS == 640, "one CTA shape");
 
 __device__ __forceinline__ int mixed_group(const MixedArgs& M) {

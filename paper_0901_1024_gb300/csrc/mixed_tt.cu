@@ -11,10 +11,8 @@ namespace dgdev {
 
 namespace {
 
-template <int N> constexpr int tt_smem() {
-  return TtDims<N>::SMEM > 120 * 1024 ? TtDims<N>::SMEM : 120 * 1024;
-}
-constexpr int kMixedTtSmem = tt_smem<5>() > tt_smem<6>() ? tt_smem<5>() : tt_smem<6>();
+constexpr int kMixedTtSmem = tc_smem(512, TtDims<5>::SMEM > TtDims<6>::SMEM ? TtDims<5>::SMEM
+                                                                             : TtDims<6>::SMEM);
 static_assert(TtDims<5>::THREADS == TtDims<6>::THREADS, "one CTA shape");
 
 __global__ void __launch_bounds__(TtDims<6>::THREADS, 1)

@@ -118,6 +118,7 @@ template <int N, bool PAIR = false> struct TcDims {
                 OFF_TAB % 16 == 0, "alignment");
   static_assert((G_FLOATS * 4) % 16 == 0, "geometry block must be a 16-byte multiple");
   static_assert(SMEM <= (PAIR ? 112 : 226) * 1024, "shared memory budget");
+  static_assert(TMEM == 256 || TMEM == 512, "tc_smem");
 };
 
 static_assert(tc_b_bytes(4) == 2 * TcDims<4>::B_BYTES, "B buffer size formula");
@@ -828,9 +829,8 @@ cudaError_t launch_tc_stage_form(bool rk, const StageArgs& a, int num_sms, cudaS
                         : tc_stage_kernel<N, true, false, PAIR>)
                  : (ext ? tc_stage_kernel<N, false, true, PAIR>
                         : tc_stage_kernel<N, false, false, PAIR>);
-  // at least 120 KB of shared memory: never two CTAs (each takes all 512
-  // tensor-memory columns) on one SM; PAIR: at least 80 KB, never three
-  constexpr int least = (PAIR ? 80 : 120) * 1024, smem = D::SMEM > least ? D::SMEM : least;
+  constexpr int smem = tc_smem(D::TMEM, D::SMEM);
+  static_assert(!PAIR || 2 * (smem + kCtaSmem) <= kSmSmem, "two CTAs an SM");
   bool& done = attr[rk ? 1 : 0][ext ? 1 : 0][dev];
   if (!done) {
     err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);

@@ -763,9 +763,7 @@ cudaError_t launch_tt_stage_n(bool rk, const StageArgs& a, int num_sms, cudaStre
   const bool ext = a.mat || a.absorbing;
   auto kern = rk ? (ext ? tt_stage_kernel<N, true, true> : tt_stage_kernel<N, true, false>)
                  : (ext ? tt_stage_kernel<N, false, true> : tt_stage_kernel<N, false, false>);
-  // at least 120 KB of shared memory: never two CTAs (each takes all 512
-  // tensor-memory columns) on one SM
-  constexpr int smem = D::SMEM > 120 * 1024 ? D::SMEM : 120 * 1024;
+  constexpr int smem = tc_smem(512, D::SMEM);
   bool& done = attr[rk ? 1 : 0][ext ? 1 : 0][dev];
   if (!done) {
     err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);

@@ -1,0 +1,55 @@
+"""What the tensor-core stage kernels ask of an SM, from the headers by a host program:
+no two CTAs that could share an SM may want more tensor memory than it has, since a CTA
+signals the next kernel before it allocates (launch.cuh)."""
+from __future__ import annotations
+
+import itertools
+import os
+import subprocess
+
+import pytest
+
+from paper_0901_1024_gb300 import build as b
+
+PROGRAM = r"""
+#include <cstdio>
+#include "tc_stage.cuh"
+#include "tc_stage_t.cuh"
+using namespace dgdev;
+template <class D> void form(const char* name, int columns) {
+  std::printf("%s %d %d\n", name, columns, tc_smem(columns, D::SMEM));
+}
+int main() {
+  form<TcDims<1>>("N1", TcDims<1>::TMEM);
+  form<TcDims<2>>("N2", TcDims<2>::TMEM);
+  form<TcDims<2, true>>("N2pair", TcDims<2, true>::TMEM);
+  form<TcDims<3>>("N3", TcDims<3>::TMEM);
+  form<TcDims<3, true>>("N3pair", TcDims<3, true>::TMEM);
+  form<TcDims<4>>("N4", TcDims<4>::TMEM);
+  form<TtDims<5>>("N5", 512);
+  form<TtDims<6>>("N6", 512);
+  form<TtDims<7>>("N7", 512);
+}
+"""
+
+SM_SMEM, CTA_SMEM, SM_COLUMNS = 228 * 1024, 1024, 512
+
+
+@pytest.fixture(scope="module")
+def forms(tmp_path_factory):
+    d = tmp_path_factory.mktemp("footprints")
+    src, exe = os.path.join(d, "f.cu"), os.path.join(d, "f")
+    with open(src, "w") as f:
+        f.write(PROGRAM)
+    subprocess.run([b._nvcc(), *b.ARCH, *b.FLAGS, src, "-o", exe], check=True, capture_output=True)
+    out = subprocess.run([exe], check=True, capture_output=True, text=True).stdout
+    return {n: (int(c), int(s)) for n, c, s in (line.split() for line in out.splitlines())}
+
+
+def test_ctas_that_fit_an_sm_fit_its_tensor_memory(forms):
+    for k in (2, 3):
+        for group in itertools.combinations_with_replacement(forms.values(), k):
+            if sum(s + CTA_SMEM for _, s in group) <= SM_SMEM:
+                assert sum(c for c, _ in group) <= SM_COLUMNS
+    for n in ("N2pair", "N3pair"):             # and the paired forms do fit twice
+        assert 2 * (forms[n][1] + CTA_SMEM) <= SM_SMEM
