@@ -97,7 +97,7 @@ template <int N> struct EnergyShape {
   static_assert(BYTES <= 227 * 1024, "shared memory");
 };
 
-template <int N, bool VEC>
+template <int N, bool VEC, class Index>
 __global__ void __launch_bounds__(EnergyShape<N>::THREADS, EnergyShape<N>::MIN_BLOCKS)
 energy_tile_kernel(const EnergyArgs A) {
   using S = EnergyShape<N>;
@@ -113,14 +113,14 @@ energy_tile_kernel(const EnergyArgs A) {
   if constexpr (NP4 != NP)                             // padding columns stay zero
     for (int i = tid; i < ROWS * (NP4 - NP); i += TH)
       sU[i / (NP4 - NP) * NP4 + NP + i % (NP4 - NP)] = 0.f;
-  const unsigned Kr = unsigned(A.k1 - A.k0), rows = 6u * Kr;   // rows (c, k): c Kr + (k - k0)
+  const Index rows = Index(energy_rows(A.k0, A.k1)), step = Index(gridDim.x) * ROWS;
   double acc = 0.0;
-  for (unsigned r0 = blockIdx.x * ROWS; r0 < rows; r0 += gridDim.x * ROWS) {
-    const int nr = int(min(rows - r0, unsigned(ROWS)));
+  for (Index r0 = Index(blockIdx.x) * ROWS; r0 < rows; r0 += step) {
+    const int nr = int(min(rows - r0, Index(ROWS)));
     __syncthreads();                                   // the previous pass is consumed
     for (int i = tid; i < nr; i += TH) {
-      const unsigned g = r0 + i, c = g / Kr;
-      const int64_t k = A.k0 + int64_t(g - c * Kr);
+      const auto [c, kr] = energy_row<Index>(r0 + i, A.k0, A.k1);
+      const int64_t k = A.k0 + kr;
       sRow[i] = (int64_t(c) * A.K + k) * NP;
       float wgt = __ldg(A.J + k);
       if (A.mat) {
@@ -226,7 +226,7 @@ __global__ void energy_finalize(const double* partials, int n, double* result) {
 // packed triangle in shared memory.  Reading the fields bounds it; staging rows for a
 // product this small cost more than it saved (a dg_energy call, staged before and now:
 // N = 1, 705 894 tets 121 -> 64 us; N = 2, 279 936 tets 83 -> 50 us).
-template <int NP, bool VEC>
+template <int NP, bool VEC, class Index>
 __global__ void __launch_bounds__(256) energy_row_kernel(const EnergyArgs A) {
   constexpr int NT = NP * (NP + 1) / 2, NT4 = (NT + 3) & ~3;
   __shared__ __align__(16) float sT[NT4];              // rows i: T_ii, T_i+1,i, ...
@@ -236,12 +236,12 @@ __global__ void __launch_bounds__(256) energy_row_kernel(const EnergyArgs A) {
     sT[x] = __ldg(A.T + (i + o) * 32 + i);
   }
   __syncthreads();
-  const unsigned Kr = unsigned(A.k1 - A.k0), rows = 6u * Kr;
+  const Index rows = Index(energy_rows(A.k0, A.k1)), step = Index(gridDim.x) * 256;
   double acc = 0.0;
 #pragma unroll 2
-  for (unsigned g = blockIdx.x * 256 + threadIdx.x; g < rows; g += gridDim.x * 256) {
-    const unsigned c = g / Kr;
-    const int64_t k = A.k0 + int64_t(g - c * Kr);
+  for (Index g = Index(blockIdx.x) * 256 + threadIdx.x; g < rows; g += step) {
+    const auto [c, kr] = energy_row<Index>(g, A.k0, A.k1);
+    const int64_t k = A.k0 + kr;
     const float* row = A.u + (int64_t(c) * A.K + k) * NP;
     float u[NP];
     if constexpr (VEC) {
@@ -287,9 +287,12 @@ int energy_grid(int num_sms) { return 8 * num_sms; }
 
 template <int NP, bool VEC>
 static cudaError_t launch_energy_row(const EnergyArgs& a, int num_sms, int* grid, cudaStream_t s) {
-  const int64_t blocks = (6 * int64_t(a.k1 - a.k0) + 255) / 256;
+  const int64_t blocks = (energy_rows(a.k0, a.k1) + 255) / 256;
   *grid = int(std::min<int64_t>(blocks, energy_grid(num_sms)));
-  energy_row_kernel<NP, VEC><<<*grid, 256, 0, s>>>(a);
+  if (energy_index32(energy_rows(a.k0, a.k1), int64_t(*grid) * 256))
+    energy_row_kernel<NP, VEC, unsigned><<<*grid, 256, 0, s>>>(a);
+  else
+    energy_row_kernel<NP, VEC, int64_t><<<*grid, 256, 0, s>>>(a);
   return cudaGetLastError();
 }
 
@@ -298,14 +301,16 @@ static cudaError_t launch_energy_n(const EnergyArgs& a, int num_sms, int* grid, 
   using S = EnergyShape<N>;
   // 16-byte copies where every row starts on a 16-byte boundary
   const bool vec = S::NP % 4 == 0 && reinterpret_cast<uintptr_t>(a.u) % 16 == 0;
-  auto kern = energy_tile_kernel<N, false>;
+  // (the row numbers of meshes past 32 bits: 4-byte copies serve)
+  const bool i32 = energy_index32(energy_rows(a.k0, a.k1), int64_t(energy_grid(num_sms)) * S::ROWS);
+  auto kern = i32 ? energy_tile_kernel<N, false, unsigned> : energy_tile_kernel<N, false, int64_t>;
   if constexpr (S::NP % 4 == 0)
-    if (vec) kern = energy_tile_kernel<N, true>;
-  static int occ[2][16] = {};                          // [vec][device]: blocks per SM
+    if (vec && i32) kern = energy_tile_kernel<N, true, unsigned>;
+  static int occ[3][16] = {};                          // [form][device]: blocks per SM
   int dev = 0;
   cudaError_t err = cudaGetDevice(&dev);
   if (err != cudaSuccess) return err;
-  int& o = occ[vec ? 1 : 0][dev & 15];
+  int& o = occ[!i32 ? 2 : vec ? 1 : 0][dev & 15];
   if (o == 0) {
     err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, S::BYTES);
     if (err != cudaSuccess) return err;
@@ -314,7 +319,7 @@ static cudaError_t launch_energy_n(const EnergyArgs& a, int num_sms, int* grid, 
     if (err != cudaSuccess) return err;
     o = n < 1 ? 1 : n > 8 ? 8 : n;
   }
-  const int64_t passes = (6 * int64_t(a.k1 - a.k0) + S::ROWS - 1) / S::ROWS;
+  const int64_t passes = (energy_rows(a.k0, a.k1) + S::ROWS - 1) / S::ROWS;
   *grid = int(std::min<int64_t>(passes, int64_t(num_sms) * o));
   kern<<<*grid, S::THREADS, S::BYTES, s>>>(a);
   return cudaGetLastError();
