@@ -816,6 +816,12 @@ tc_stage_kernel(const __grid_constant__ StageArgs A) {
   tc_stage_body<N, RK, EXT, PAIR>(A, int(blockIdx.x), int(gridDim.x));
 }
 
+// Up to one tile an SM, a CTA asks for enough shared memory to have its SM to itself: two
+// paired CTAs on one SM while others idle finish later (order 2, 800 to 3 020 tetrahedra
+// 5.0-5.3 us a stage side by side, 4.5-4.6 alone, 4.7-4.8 in the one-CTA form; with
+// materials 5.7 and 4.7).
+constexpr bool tc_cta_alone(int tiles, int sms) { return tiles <= sms; }
+
 template <int N, bool PAIR>
 cudaError_t launch_tc_stage_form(bool rk, const StageArgs& a, int num_sms, cudaStream_t s) {
   using D = TcDims<N, PAIR>;
@@ -829,11 +835,12 @@ cudaError_t launch_tc_stage_form(bool rk, const StageArgs& a, int num_sms, cudaS
                         : tc_stage_kernel<N, true, false, PAIR>)
                  : (ext ? tc_stage_kernel<N, false, true, PAIR>
                         : tc_stage_kernel<N, false, false, PAIR>);
-  constexpr int smem = tc_smem(D::TMEM, D::SMEM);
-  static_assert(!PAIR || 2 * (smem + kCtaSmem) <= kSmSmem, "two CTAs an SM");
+  constexpr int shared = tc_smem(D::TMEM, D::SMEM), alone = tc_smem(512, D::SMEM);
+  static_assert(!PAIR || 2 * (shared + kCtaSmem) <= kSmSmem, "two CTAs an SM");
+  const int smem = tc_cta_alone(a.num_tiles, num_sms) ? alone : shared;
   bool& done = attr[rk ? 1 : 0][ext ? 1 : 0][dev];
   if (!done) {
-    err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
+    err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, alone);
     if (err != cudaSuccess) return err;
     done = true;
   }

@@ -29,6 +29,10 @@ int main() {
   form<TtDims<5>>("N5", 512);
   form<TtDims<6>>("N6", 512);
   form<TtDims<7>>("N7", 512);
+  // shared memory of the launch of 1, 65, 152, 153 and 14 000 tiles on 152 SMs
+  for (int tiles : {1, 65, 152, 153, 14000})
+    std::printf("alone%d %d %d\n", tiles, tc_cta_alone(tiles, 152) ? 1 : 0,
+                tc_cta_alone(tiles, 152) ? tc_smem(512, TcDims<2, true>::SMEM) : 0);
 }
 """
 
@@ -46,10 +50,22 @@ def forms(tmp_path_factory):
     return {n: (int(c), int(s)) for n, c, s in (line.split() for line in out.splitlines())}
 
 
+def kernels(forms):
+    return [v for n, v in forms.items() if n.startswith("N")]
+
+
 def test_ctas_that_fit_an_sm_fit_its_tensor_memory(forms):
     for k in (2, 3):
-        for group in itertools.combinations_with_replacement(forms.values(), k):
+        for group in itertools.combinations_with_replacement(kernels(forms), k):
             if sum(s + CTA_SMEM for _, s in group) <= SM_SMEM:
                 assert sum(c for c, _ in group) <= SM_COLUMNS
     for n in ("N2pair", "N3pair"):             # and the paired forms do fit twice
         assert 2 * (forms[n][1] + CTA_SMEM) <= SM_SMEM
+
+
+def test_a_wave_or_less_has_one_cta_an_sm(forms):
+    """Up to one tile an SM no SM may take two CTAs while another idles."""
+    for tiles in (1, 65, 152):
+        alone, smem = forms[f"alone{tiles}"]
+        assert alone == 1 and 2 * (smem + CTA_SMEM) > SM_SMEM
+    assert forms["alone153"][0] == 0 and forms["alone14000"][0] == 0
