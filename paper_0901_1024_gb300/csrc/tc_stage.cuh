@@ -849,17 +849,27 @@ cudaError_t launch_tc_stage_form(bool rk, const StageArgs& a, int num_sms, cudaS
   return launch_pdl(kern, grid, D::THREADS, smem, s, a);
 }
 
+// Whether a launch of `tiles` tiles runs two CTAs an SM (launched alone; a mixed launch has
+// one CTA shape).  Order 2 always (279 936 tetrahedra 176 -> 120 us a stage, 384 4.8 -> 4.5).
+// Order 3 from one tile an SM on (146 334 tetrahedra 130 -> 117 us, 6 000 9.0 -> 7.9), but not
+// where the last round has a tile for more than half of the SMs but not for all: one CTA
+// of a pair then works alone, at the pace of two (400 tiles 12.7 us
+// against 11.4 in one CTA an SM, 740 17.3 against 16.6, with materials 13.3 and 11.9, 18.3 and
+// 17.3; 360 tiles 11.2 and 11.4, 456 11.3 and 11.5, 680 15.4 and 16.5; from seven rounds on within 1 %).
+// Order 1 on request and order 4 (whose tiles do not fit twice) as one.
+constexpr bool tc_paired(int N, int tiles, int sms) {
+  if (N != 3) return N == 2;
+  const int rest = tiles % (2 * sms);              // tiles of the last round of CTA pairs
+  const bool half = 2 * rest > sms && rest < sms;
+  return tiles > sms && !(half && tiles < 5 * sms);
+}
+
 template <int N>
 cudaError_t launch_tc_stage_n(bool rk, const StageArgs& a, int num_sms, cudaStream_t s) {
-  // Two CTAs an SM (launched alone; a mixed launch has one CTA shape): order 2 always (384
-  // tetrahedra 5.1 -> 4.8 us a stage, 279 936 176 -> 120 us), order 3 when an SM gets more
-  // than one tile (146 334 tetrahedra 130 -> 117 us, 3 072 8.7 -> 8.1 us, but 384, one tile
-  // a CTA, 6.1 -> 6.5 us).  Order 1 on request and order 4 (whose tiles do not fit twice)
-  // as one.
-  if constexpr (N == 2) return launch_tc_stage_form<N, true>(rk, a, num_sms, s);
-  if constexpr (N == 3)
-    if (a.num_tiles > num_sms) return launch_tc_stage_form<N, true>(rk, a, num_sms, s);
+  if constexpr (N == 2 || N == 3)
+    if (tc_paired(N, a.num_tiles, num_sms)) return launch_tc_stage_form<N, true>(rk, a, num_sms, s);
   if constexpr (N != 2) return launch_tc_stage_form<N, false>(rk, a, num_sms, s);
+  return cudaErrorInvalidValue;                    // not reached
 }
 
 }  // namespace dgdev

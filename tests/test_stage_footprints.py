@@ -33,6 +33,9 @@ int main() {
   for (int tiles : {1, 65, 152, 153, 14000})
     std::printf("alone%d %d %d\n", tiles, tc_cta_alone(tiles, 152) ? 1 : 0,
                 tc_cta_alone(tiles, 152) ? tc_smem(512, TcDims<2, true>::SMEM) : 0);
+  for (int N = 1; N <= 4; ++N)
+    for (int tiles : {1, 152, 153, 304, 360, 381, 400, 455, 456, 608, 680, 700, 759, 760, 1000, 7317})
+      std::printf("pair%d_%d %d 0\n", N, tiles, tc_paired(N, tiles, 152) ? 1 : 0);
 }
 """
 
@@ -69,3 +72,12 @@ def test_a_wave_or_less_has_one_cta_an_sm(forms):
         alone, smem = forms[f"alone{tiles}"]
         assert alone == 1 and 2 * (smem + CTA_SMEM) > SM_SMEM
     assert forms["alone153"][0] == 0 and forms["alone14000"][0] == 0
+
+
+def test_which_launches_are_paired(forms):
+    """On 152 SMs: order 2 always, order 3 where two CTAs an SM measured faster (no worse than
+    1 % slower), orders 1 and 4 never."""
+    for tiles in (1, 152, 153, 304, 360, 381, 400, 455, 456, 608, 680, 700, 759, 760, 1000, 7317):
+        assert [forms[f"pair{N}_{tiles}"][0] for N in (1, 2, 4)] == [0, 1, 0]
+        single = tiles <= 152 or 380 < tiles < 456 or 684 < tiles < 760
+        assert forms[f"pair3_{tiles}"][0] == (0 if single else 1), tiles
