@@ -225,7 +225,9 @@ __global__ void energy_finalize(const double* partials, int n, double* result) {
 // Orders 1 and 2 (4 and 10 nodes): a row per thread straight from global memory, the
 // packed triangle in shared memory.  Reading the fields bounds it; staging rows for a
 // product this small cost more than it saved (a dg_energy call, staged before and now:
-// N = 1, 705 894 tets 121 -> 64 us; N = 2, 279 936 tets 83 -> 50 us).
+// N = 1, 705 894 tets 121 -> 64 us; N = 2, 279 936 tets 83 -> 50 us).  A row sum is one
+// chain of multiply-adds at N = 1 and two at N = 2, whichever is the nearer to 64 bits (rms
+// over random rows, one chain and two: N = 1 6.57e-8 and 6.71e-8, N = 2 8.38e-8 and 8.06e-8).
 template <int NP, bool VEC, class Index>
 __global__ void __launch_bounds__(256) energy_row_kernel(const EnergyArgs A) {
   constexpr int NT = NP * (NP + 1) / 2, NT4 = (NT + 3) & ~3;
@@ -263,10 +265,13 @@ __global__ void __launch_bounds__(256) energy_row_kernel(const EnergyArgs A) {
     int x = 0;
 #pragma unroll
     for (int i = 0; i < NP; ++i) {
-      float s = 0.f;
+      float s[2] = {0.f, 0.f};                         // order 2: every other column apart
 #pragma unroll
-      for (int j = i; j < NP; ++j) s = fmaf(sT[x++], u[j], s);
-      e = fmaf(u[i], s, e);
+      for (int j = i; j < NP; ++j) {
+        float& t = s[NP > 4 ? (j - i) & 1 : 0];
+        t = fmaf(sT[x++], u[j], t);
+      }
+      e = fmaf(u[i], NP > 4 ? s[0] + s[1] : s[0], e);
     }
     acc += double(wgt) * double(e);
   }
