@@ -255,26 +255,38 @@ class Server:
         return (self.torch.cuda.current_device(), N,
                 min(3, int(math.log10(max(K, 1))) - 2))     # <1e3, <1e4, <1e5, more
 
+    def _time_steps(self, step):
+        """Milliseconds of 3 calls of `step` on the server's stream, after 2 untimed ones."""
+        torch = self.torch
+        for _ in range(2):
+            step()
+        e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
+        e0.record(self.stream)
+        for _ in range(3):
+            step()
+        e1.record(self.stream)
+        e1.synchronize()
+        return e0.elapsed_time(e1)
+
     def _time_impl(self, N, solves, impl, shape=0):
         """Milliseconds of 3 steps of a scratch pack of `solves` on `impl` with
         tile shape `shape`; the pack is released before returning."""
         torch = self.torch
         self._charge(sum(s.bytes for s in solves))
         p = _Pack(torch, N, solves, None, self._pad_mesh(N), impl, False, self.stream, shape)
-        for _ in range(2):                       # warm-up
-            p.step()
-        e0, e1 = torch.cuda.Event(enable_timing=True), torch.cuda.Event(enable_timing=True)
-        e0.record(self.stream)
-        for _ in range(3):
-            p.step()
-        e1.record(self.stream)
-        e1.synchronize()
-        ms = e0.elapsed_time(e1)
+        ms = self._time_steps(p.step)
         if impl == Mesh.STAGE_TC and N <= 7:
-            # one tile's cost on one SM: stage time x CTAs in use / tiles
+            # one tile's cost on one SM of a shared launch: stage time x CTAs in use / tiles.
+            # Orders 1..6 are timed in one, since a pack of order 2 or 3 launched alone may run
+            # two CTAs an SM and a shared launch does not (order 2: its tiles cost 1.47x as
+            # much there); order 7 is launched alone in any case.
+            if N <= 6:
+                ms_shared = self._time_steps(lambda: self._stages_mixed([p], p.parity))
+            else:
+                ms_shared = ms
             tiles = -(-p.K // (20 if N <= 4 else 8))
             sms = torch.cuda.get_device_properties(torch.cuda.current_device()).multi_processor_count
-            self._cost[self._tune_key(N, solves)] = ms / 15 * min(tiles, sms) / tiles
+            self._cost[self._tune_key(N, solves)] = ms_shared / 15 * min(tiles, sms) / tiles
         p.release()
         self._charge(-sum(s.bytes for s in solves))
         return ms
