@@ -53,7 +53,6 @@ namespace dgdev {
 // Their tiles are so small that the chain of barriers, not the work, takes the time (4 k
 // cycles a tile at order 2, a third of the issue slots used); two chains share the SM.
 template <int N, bool PAIR = false> struct TcDims {
-  static constexpr int ORDER = N;
   static constexpr int Np = (N + 1) * (N + 2) * (N + 3) / 6;
   static constexpr int Nfp = (N + 1) * (N + 2) / 2;
   static constexpr int NF = 4 * Nfp;
@@ -245,7 +244,6 @@ struct GRow {
   const float* sg;
   float* sBound;
   float* sScale;
-  int us;                 // field stride of su
   int t, row, rc, re, o, fa, fb;
   float sgn;
   bool live;
@@ -262,8 +260,8 @@ __device__ __forceinline__ void build_g_half(const GRow& g, int role) {
   constexpr int E = D::E, Np = D::Np;
   float2 ua[NPH], ub[NPH];
   float umax = 0.f;
-  const float* pa = g.su + g.fa * g.us + g.re * Np;
-  const float* pb = g.su + g.fb * g.us + g.re * Np;
+  const float* pa = g.su + (g.fa * E + g.re) * Np;
+  const float* pb = g.su + (g.fb * E + g.re) * Np;
 #pragma unroll
   for (int i = 0; i < NPH; ++i) {
     const int j = 2 * (P0 + i);
@@ -358,14 +356,14 @@ __device__ __forceinline__ uint32_t tc_item(int idx, int elems, const unsigned c
 
 // Flux extraction (Alg. 3) of the face nodes `item` (decoded e | m << 5 | f << 12 |
 // idM << 14, bit 31: none) of the tile starting at element k0 with Ev valid
-// elements, fields su (stride us) and geometry sg in shared memory: classify, gather the
+// elements, fields su and geometry sg in shared memory: classify, gather the
 // neighbour values outside the tile, form the upwind fluxes (PEC ghost state on
 // walls, zero exterior state on absorbing faces) and store them at
 // dst + (c * CS + e - E0) * FSTR + m for field c of element e (E0 <= e < E0 + CS).
 template <int N, bool EXT, int NI>
 __device__ __forceinline__ void tc_flux_items(const uint32_t (&item)[NI], const StageArgs& A,
-                                              int k0, int Ev, const float* su, int us,
-                                              const float* sg, float* dst, int CS, int E0) {
+                                              int k0, int Ev, const float* su, const float* sg,
+                                              float* dst, int CS, int E0) {
   using D = TcDims<N>;
   constexpr int E = D::E, Np = D::Np, NF = D::NF, FSTR = D::FSTR;
   const int K = A.K;
@@ -426,11 +424,11 @@ __device__ __forceinline__ void tc_flux_items(const uint32_t (&item)[NI], const 
       const int idM = (it >> 14) & 63;
       const float* pp = kind == 3u ? dst + (e - E0) * FSTR + m
                                    : su + (EXT ? (info[q] >> 2) & 0x1FFFFFFFu : info[q] >> 2);
-      const int ps = kind == 3u ? CS * FSTR : us;
+      const int ps = kind == 3u ? CS * FSTR : E * Np;
       const bool zero_ext = EXT && (info[q] >> 31);          // absorbing: u+ = 0
 #pragma unroll
       for (int c = 0; c < 6; ++c) {
-        uM[q][c] = su[c * us + e * Np + idM];
+        uM[q][c] = su[c * E * Np + e * Np + idM];
         up[q][c] = zero_ext ? 0.f : pp[c * ps];
       }
 #pragma unroll
@@ -517,7 +515,6 @@ __device__ __forceinline__ void tc_stage_body(const StageArgs& A, const int cta,
 
   const int tid = threadIdx.x, warp = tid >> 5, lane = tid & 31;
   const int K = A.K;
-  constexpr int us = E * Np;                       // field stride in shared memory
   const int ntiles = (A.num_tiles - cta + ncta - 1) / ncta;
   const int base = A.tile0 + cta;                  // this CTA's first tile of the mesh
   if (ntiles <= 0) return;
@@ -580,7 +577,7 @@ __device__ __forceinline__ void tc_stage_body(const StageArgs& A, const int cta,
         const int slot = t % D::NSU;
         const int k0t = (base + t * ncta) * E, Evt = min(E, K - k0t);
         wait_or_flag(&s_u_full[slot], (t / D::NSU) & 1, A.status);
-        tc_flux_items<N, EXT, D::EITEMS>(eitem, A, k0t, Evt, sU + slot * D::U_FLOATS, us,
+        tc_flux_items<N, EXT, D::EITEMS>(eitem, A, k0t, Evt, sU + slot * D::U_FLOATS,
                                          sG + slot * D::G_FLOATS, sF2 + (t & 1) * D::F2_FLOATS,
                                          E - D::E0, D::E0);
       }
@@ -606,11 +603,9 @@ __device__ __forceinline__ void tc_stage_body(const StageArgs& A, const int cta,
         const uint64_t b_lo = b_hi + uint64_t(D::B_BYTES >> 4);
 #pragma unroll
         for (int i = 0; i < 3 * D::KSTEPS; ++i) {
-          // passes: hi.hi, hi.lo, lo.hi
-          const int q = i / D::KSTEPS, ks = i - q * D::KSTEPS;
-          const bool al = q == 2, bl = q == 1;
-          const uint64_t bd = (bl ? b_lo : b_hi) + uint64_t((ks * 2 * LBO) >> 4);
-          const uint32_t ad = a_base + (al ? D::ACOLS : 0) + ks * 8;
+          const int p = i / D::KSTEPS, ks = i - p * D::KSTEPS;   // passes: hi.hi, hi.lo, lo.hi
+          const uint64_t bd = (p == 1 ? b_lo : b_hi) + uint64_t((ks * 2 * LBO) >> 4);
+          const uint32_t ad = a_base + (p == 2 ? D::ACOLS : 0) + ks * 8;
           tc::mma_f16_ts_warp(d_acc, ad, bd, IDESC, i > 0 ? 1u : 0u);
         }
         tc::mma_commit_warp(&s_mma_done[buf]);
@@ -655,8 +650,8 @@ __device__ __forceinline__ void tc_stage_body(const StageArgs& A, const int cta,
             inv *= rc < 3 ? w.x : w.y;
           }
           const float dte = RK && A.dt_elem ? __ldg(A.dt_elem + k0 + re) : A.dt;
-          float* pr = sr + rc * us + re * Np;
-          float* pu = su + rc * us + re * Np;
+          float* pr = sr + (rc * E + re) * Np;
+          float* pu = su + (rc * E + re) * Np;
           // u and res share one shared array, so every batch is loaded before any
           // of its stores (the compiler cannot move loads across them)
           // (batches of 8 at order 4: 99.6 us a stage on 82 944 tetrahedra, of 12 101.2, of 18
@@ -753,10 +748,10 @@ __device__ __forceinline__ void tc_stage_body(const StageArgs& A, const int cta,
       for (int q = 0; q < D::ITEMS; q += 2) {         // two items' operands in registers
         if (q + 1 < D::ITEMS) {
           const uint32_t it[2] = {item[q], item[q + 1]};
-          tc_flux_items<N, EXT, 2>(it, A, k0, Ev, su, us, sg, F, E, 0);
+          tc_flux_items<N, EXT, 2>(it, A, k0, Ev, su, sg, F, E, 0);
         } else {
           const uint32_t it[1] = {item[q]};
-          tc_flux_items<N, EXT, 1>(it, A, k0, Ev, su, us, sg, F, E, 0);
+          tc_flux_items<N, EXT, 1>(it, A, k0, Ev, su, sg, F, E, 0);
         }
       }
       // The flux buffer is complete once every producer has stored its items:
@@ -789,7 +784,7 @@ __device__ __forceinline__ void tc_stage_body(const StageArgs& A, const int cta,
         // roles 0 and 1 split the node range: node pairs [0, H) and [H, KB/2) of
         // all three g blocks, each loading only its half of the two curl fields
         constexpr int H = (D::KB / 2 + 1) / 2;
-        const GRow gr{su, sg, sBound, sScale, us, t, row, rc, re, o, fa, fb, sgn, live, a_hi, a_lo,
+        const GRow gr{su, sg, sBound, sScale, t, row, rc, re, o, fa, fb, sgn, live, a_hi, a_lo,
                       &s_mma_done[(t - D::ABUF) & 1], A.status};
         if constexpr (PAIR)
           build_g_half<D, 0, D::KB / 2>(gr, 0);
@@ -876,5 +871,5 @@ cudaError_t launch_tc_stage_n(bool rk, const StageArgs& a, int num_sms, cudaStre
 
 #define DG_INSTANTIATE_TC_STAGE(NN)                                                        \
   namespace dgdev {                                                                         \
-  template cudaError_t launch_tc_stage_n<NN>(bool, const StageArgs&, int, cudaStream_t);   \
+  template cudaError_t launch_tc_stage_n<NN>(bool, const StageArgs&, int, cudaStream_t);    \
   }
