@@ -1096,7 +1096,7 @@ int device_wait_selftest(dg_mesh* m, uint32_t polls, double* seconds, std::strin
 static int energy_impl(dg_mesh* m, const float* u, double* out, cudaStream_t s,
                        std::string& err, int64_t k0 = 0, int64_t k1 = -1) {
   DeviceState* d = m->dev;
-  dgdev::EnergyArgs a{u, d->T, d->J, static_cast<int>(d->K), d->Np, d->partials, d->result,
+  dgdev::EnergyArgs a{u, d->T, d->J, static_cast<int>(d->K), d->partials, d->result,
                       static_cast<int>(k0), static_cast<int>(k1 < 0 ? d->K : k1), d->mat};
   int grid = 0;
   DG_CUDA(traced(m, s, 2, [&] {

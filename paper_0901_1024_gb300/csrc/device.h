@@ -151,7 +151,7 @@ struct EnergyArgs {
   const float* u;      // [6][K][Np]
   const float* T;      // weighted triangle of M (device.cu, energy kernel)
   const float* J;      // [K]
-  int K, Np;
+  int K;
   double* partials;    // [blocks of the launch <= energy_grid]
   double* result;      // [1]
   int k0, k1;          // elements k0 <= k < k1 (0, K: the whole mesh)
