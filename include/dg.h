@@ -255,8 +255,9 @@ int dg_rk_stage_range(dg_mesh* mesh, const float* u_in, float* u_out, float* res
                       double dt, int64_t k0, int64_t k1, void* stream);
 
 /*
- * Self-test of failure detection in the tensor-core stages: every mbarrier
- * wait of those kernels is bounded and, when it runs out, sets the mesh's
+ * Self-test of failure detection in the stage kernels: every mbarrier wait of
+ * theirs (the tensor-core stages, and the FP32 stage of orders 8 and 9 for its
+ * operator's copies) is bounded and, when it runs out, sets the mesh's
  * pipeline status word, which dg_energy, dg_energy_range and dg_step_host read
  * (and clear) after their synchronisation and report as DG_ERR_CUDA.  This
  * call runs the same bounded wait, limited to `polls` polls, in a one-warp

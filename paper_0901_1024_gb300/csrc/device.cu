@@ -1068,7 +1068,7 @@ int device_step(dg_mesh* m, float* u, float* res, double dt, int nsteps, void* s
 static int report_status(dg_mesh* m, int st, std::string& err) {
   if (st != 0) {
     DG_CUDA(cudaMemset(m->dev->status, 0, sizeof(int)), "cudaMemset");
-    err = "tensor-core stage: an MMA completion wait timed out (results invalid)";
+    err = "stage kernel: a wait for a copy or for tensor-core results timed out (results invalid)";
     return DG_ERR_CUDA;
   }
   return DG_OK;

@@ -77,7 +77,7 @@ struct StageArgs {
                             // K-major shared-memory layout, orders 5..7 as tensor-memory rows
   float tc_inv_bscale;      // 1 / (power-of-two scale applied to [Dr Ds Dt LIFT])
   const void* wide;         // register-tiled FP32 stage: packed operator chunks
-  int* status;              // set to 1 if an MMA completion wait timed out
+  int* status;              // set to 1 if a stage kernel's bounded wait ran out
   int absorbing;            // 1 if any boundary face is absorbing (code kAbsorbingCode)
 };
 
