@@ -958,8 +958,9 @@ int device_stage(dg_mesh* m, const float* u_in, float* u_out, float* res, int st
 }
 
 // Default cost of one tile on one SM in microseconds, orders 1..6 on the
-// tensor cores (GB300: stage time x CTAs / tiles of the order sweep), used to
-// split a mixed launch's CTAs when the caller gives no costs.
+// tensor cores in the one-CTA form that a mixed launch runs (GB300: stage time x
+// SMs / tiles at ~1.7e7 unknowns), used to split a mixed launch's CTAs when the
+// caller gives no costs.
 static double default_tile_cost(int N) {
   static const double c[7] = {1.0, 1.6, 1.9, 2.7, 3.6, 3.1, 3.9};
   return N >= 1 && N <= 6 ? c[N] : 1.0;

@@ -16,8 +16,9 @@
 // and B = [Dr Ds Dt LIFT] scaled by a power of two; both scales are removed in
 // the epilogue.
 //
-// One persistent CTA per SM (all 512 tensor-memory columns), two warp groups
-// working on different tiles at once, linked by mbarriers:
+// One persistent CTA per SM (all 512 tensor-memory columns), or at orders 2 and 3 two of
+// half the columns (PAIR below; tc_paired() at the end says where), with two warp groups
+// working on different tiles at once, linked by mbarriers.  The one-CTA form:
 //   * producer warps (16): together they compute the fluxes of tile t (flux
 //     extraction, Alg. 3 of the paper; up to 2 face nodes per thread; at N = 4
 //     the face nodes of the tile's last 3 elements are done one tile earlier by
@@ -38,7 +39,9 @@
 //     res <- a res + dt rhs, u <- u + b res in place in shared memory, and
 //     bulk copies write u_out and res back.
 // Fields and geometry arrive by bulk copies four tiles ahead into a 5-slot
-// ring; the RK register one tile ahead into a 2-slot ring.
+// ring; the RK register one tile ahead into a 2-slot ring.  The paired form has 8
+// producer warps (role 0 the g blocks, role 1 the flux block), no flux items on the
+// epilogue warps, and at order 3 a 4-slot ring and one A buffer.
 #pragma once
 
 #include <cuda_runtime.h>
@@ -94,7 +97,7 @@ template <int N, bool PAIR = false> struct TcDims {
   static constexpr int EPI = (E - E0) * NF;              // face nodes of the epilogue threads
   static constexpr int EITEMS = EPI ? (EPI + 95) / 96 : 1;   // per thread of warps 1..3
   static constexpr int FCOUNT = PRODUCERS + (EPI ? 128 : 0);  // threads at the flux barrier
-  static constexpr int NSU = PAIR && N == 3 ? 4 : 5, NSR = 2;              // ring slots: fields+geometry, RK register
+  static constexpr int NSU = PAIR && N == 3 ? 4 : 5, NSR = 2;   // ring slots: fields+geometry, RK register
   // shared memory (bytes)
   static constexpr int U_FLOATS = 6 * E * Np;         // one tile of one state array
   static constexpr int G_FLOATS = tc_geo_floats(N);  // word-major [w][E], node bytes
