@@ -108,12 +108,22 @@ KERNEL_SOURCES = {
     "tc": ("tc_stage.cuh", "tcgen05.cuh", "launch.cuh", "device.h"),      # tensor cores, N <= 4
     "tt": ("tc_stage_t.cuh", "tc_stage.cuh", "tcgen05.cuh", "launch.cuh",
            "device.h"),                                                   # tensor cores, N = 5..7
-    "fp32": ("stage_kernel.cuh", "tcgen05.cuh", "launch.cuh", "device.h"),  # CUDA cores
+    "fp32": ("stage_kernel.cuh", "stage_wide.cuh", "direct_stage.cuh", "tcgen05.cuh",
+             "launch.cuh", "device.h"),                                   # CUDA cores
 }
 
 
 def kernel_family(N, tc_path):
     return ("tc" if N <= 4 else "tt") if tc_path else "fp32"
+
+
+def kernel_name(N, tc_path):
+    """The stage kernel of order N at the benchmark's sizes, for the result line."""
+    if tc_path:
+        return (f"tc_stage_kernel<N={N},RK> (tcgen05, FP16x3 split)" if N <= 4 else
+                f"tt_stage_kernel<N={N},RK> (tcgen05, FP16x3 split, operator in tensor memory)")
+    name = "direct_stage_kernel" if N == 1 else "stage_wide_kernel" if N >= 8 else "stage_kernel"
+    return f"{name}<N={N},RK> (FP32 CUDA cores)"
 
 
 def kernel_source_digest(family):
@@ -372,10 +382,7 @@ def run_ours(args):
                        "element_order": args.order, "stage_kernel": args.stage_kernel},
             "roofline": {"bound": "hbm", "achieved": achieved, "peak": peaks["hbm_gbs"], "unit": "GB/s",
                          "frac": achieved / peaks["hbm_gbs"], "traffic": traffic,
-                         "kernel": ((f"tc_stage_kernel<N={w['N']},RK> (tcgen05, FP16x3 split)" if w["N"] <= 4
-                                     else f"tt_stage_kernel<N={w['N']},RK> (tcgen05, FP16x3 split, "
-                                          "operator in tensor memory)") if tc_path
-                                    else f"stage_kernel<N={w['N']},RK> (FP32 CUDA cores)"),
+                         "kernel": kernel_name(w["N"], tc_path),
                          "algorithmic_bytes_per_launch": algo_bytes,
                          "avg_launch_ms": avg_stage_s * 1e3, "launches_timed": stage_launches,
                          "avg_launch_source": avg_src,
