@@ -12,9 +12,11 @@
 //     shared-memory buffers, one bulk copy a chunk, the next chunk's under way while one
 //     is multiplied; LIFT follows through the same buffers.
 // Measured (~1.7e7 unknowns, before and after): N = 8 1014 -> 720-730 us, N = 9 1214 -> 940-950
-// us; 37 and 40 % of the FP32 peak, the loop held up by register-bank conflicts (dispatch
-// stalls).  Two CTAs an SM with half the tile 732 / 965 us, packed FP32x2 multiply-adds
-// with 8 rows a thread 747 / 957 us.
+// us; 37 and 40 % of the FP32 peak.  Half of the cycles issue nothing (N = 8: issue 52 %, FMA
+// pipe 43 %): first for the global loads of staging, fluxes and update, which no multiply-add
+// of the CTA runs beside (long scoreboard 1.29 per issued instruction), then for register
+// banks in the loop (dispatch 0.86).  Two CTAs an SM with half the tile 732 / 965 us, packed
+// FP32x2 multiply-adds with 8 rows a thread 747 / 957 us.
 #pragma once
 
 #include <algorithm>

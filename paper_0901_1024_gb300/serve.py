@@ -217,8 +217,10 @@ class Server:
                  the tuned cost of a tile of each pack; graphs capture the five
                  shared stages of the current set of packs.  Off by default:
                  on GB300 different orders side by side in one grid measured
-                 12 % slower than one launch per order (packs of one order
-                 gain 10 %), see the benchmark's serve mode.
+                 slower than one launch per order (packs of 26 832 tets, orders
+                 2 + 4 0.31 against 0.26 ms a step, 5 + 6 0.90 against 0.79), two
+                 packs of one order 10 % faster at order 4, 3 % at 3 and 7 %
+                 slower at 2, whose own launches run two CTAs an SM.
     """
 
     def __init__(self, hbm_budget: float = 150e9, batch: bool = True, graphs: bool = True,
