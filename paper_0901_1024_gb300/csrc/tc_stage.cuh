@@ -658,8 +658,9 @@ __device__ __forceinline__ void tc_stage_body(const StageArgs& A, const int cta,
           // u and res share one shared array, so every batch is loaded before any
           // of its stores (the compiler cannot move loads across them)
           // (batches of 8 at order 4: 99.6 us a stage on 82 944 tetrahedra, of 12 101.2, of 18
-          // 100.9)
-          constexpr int CH = N == 4 ? 8 : 12;
+          // 100.9; but with absorbing faces 111.6 against 107.8 of 12, with materials 116.5
+          // against 115.6)
+          constexpr int CH = N == 4 && !EXT ? 8 : 12;
 #pragma unroll
           for (int i0 = 0; i0 < Np; i0 += CH) {
             float rv[CH], uv[CH];
