@@ -836,7 +836,7 @@ static cudaError_t launch_path(const dg_mesh* m, Path p, bool rk, const dgdev::S
         for (int f = 0; f < 4 * o.Nfp; ++f)
           o.L[i][f] = static_cast<float>(m->ops.LIFT[i * 4 * o.Nfp + f]);
       }
-      return dgdev::launch_direct_stage(rk, e, o, s);
+      return dgdev::launch_direct_stage(rk, e, o, sms, s);
     }
     case Path::tc: return dgdev::launch_tc_stage(m->N, rk, a, sms, s);
     default: return dgdev::launch_stage(m->N, rk, a, sms, s, m->stage_shape);

@@ -145,7 +145,8 @@ template <int N> struct DirectOps {
   float D[3][Np][Np];      // Dr, Ds, Dt
   float L[Np][4 * Nfp];    // LIFT
 };
-cudaError_t launch_direct_stage(bool rk, const StageArgs& a, const DirectOps<1>& o, cudaStream_t s);
+cudaError_t launch_direct_stage(bool rk, const StageArgs& a, const DirectOps<1>& o, int num_sms,
+                                cudaStream_t s);
 
 struct EnergyArgs {
   const float* u;      // [6][K][Np]

@@ -38,11 +38,27 @@ __host__ __device__ constexpr int direct_face_node(int N, int f, int j) {
 
 constexpr int kDirectThreads = 128;
 
-template <int N, bool RK, bool EXT>
+// What a mesh has beside vacuum and conducting walls: nothing, absorbing faces, materials
+// (and absorbing faces, maybe), or either as the arguments say.  The last is the fastest on
+// large meshes (705 894 tetrahedra: absorbing 86 us a stage, materials 92; told apart at
+// compile time 92 and 104, by more registers in flight and spills), but its branches keep a
+// face's loads behind the face before, which small meshes wait for.
+enum class Ext { none, absorbing, materials, any };
+// Told apart where at most every other SM has a CTA (1 296 tetrahedra: absorbing 6.6 -> 5.6 us a
+// stage, materials 6.7 -> 6.2, tiles 6.0 and 6.2; 6 000: 6.9 -> 5.9, 7.2 -> 6.5, tiles 10.1 and 10.4;
+// 10 368, 81 CTAs: 8.2 and 8.6, told apart 8.6 and 9.1).
+inline Ext direct_ext(bool materials, bool absorbing, int grid, int num_sms) {
+  if (!materials && !absorbing) return Ext::none;
+  if (2 * grid > num_sms) return Ext::any;
+  return materials ? Ext::materials : Ext::absorbing;
+}
+
+template <int N, bool RK, Ext EXT>
 __global__ void __launch_bounds__(kDirectThreads, 4)
 direct_stage_kernel(const __grid_constant__ StageArgs A, const __grid_constant__ DirectOps<N> O) {
   constexpr int Np = DirectOps<N>::Np, Nfp = DirectOps<N>::Nfp, NF = 4 * Nfp;
   constexpr int TE = tc_tile_elems(N);
+  const bool mat = EXT == Ext::materials || (EXT == Ext::any && A.mat);
   static_assert(Np == 4, "a row is one 16-byte word");
   pdl_launch_dependents();
   const int k = A.tile0 + int(blockIdx.x) * kDirectThreads + int(threadIdx.x);   // first element: tile0
@@ -73,6 +89,12 @@ direct_stage_kernel(const __grid_constant__ StageArgs A, const __grid_constant__
   }
 
   const float4* U = reinterpret_cast<const float4*>(A.u_in);
+  float wE = 1.f, wH = 1.f;                        // rhs_E / eps, rhs_H / mu
+  if constexpr (EXT == Ext::materials) {
+    const float4 w = __ldg(A.mat + size_t(k) * kMatVecs);
+    wE = w.x;
+    wH = w.y;
+  }
   float u[6][Np];
 #pragma unroll
   for (int c = 0; c < 6; ++c) {
@@ -117,7 +139,7 @@ direct_stage_kernel(const __grid_constant__ StageArgs A, const __grid_constant__
 #pragma unroll
   for (int f = 0; f < 4; ++f) {
     const unsigned code = (codes >> (8 * f)) & 0xffu;
-    const bool absorbing = EXT && code == kAbsorbingCode, wall = code == 0u || absorbing;
+    const bool absorbing = EXT != Ext::none && code == kAbsorbingCode, wall = code == 0u || absorbing;
     float n[6][Np];                                // neighbour rows (walls: the element's own)
 #pragma unroll
     for (int c = 0; c < 6; ++c) {
@@ -127,7 +149,7 @@ direct_stage_kernel(const __grid_constant__ StageArgs A, const __grid_constant__
     const float nx = __ldg(g + (10 + 4 * f) * TE), ny = __ldg(g + (11 + 4 * f) * TE);
     const float nz = __ldg(g + (12 + 4 * f) * TE), sc = 0.5f * __ldg(g + (13 + 4 * f) * TE);
     float4 cf = make_float4(1.f, 0.5f, 1.f, 0.5f);
-    if (EXT && A.mat) cf = __ldg(A.mat + size_t(k) * kMatVecs + 1 + f);
+    if (mat) cf = __ldg(A.mat + size_t(k) * kMatVecs + 1 + f);
     const float al = A.alpha;
 #pragma unroll
     for (int j = 0; j < Nfp; ++j) {
@@ -157,7 +179,7 @@ direct_stage_kernel(const __grid_constant__ StageArgs A, const __grid_constant__
       // E: -n x dH + alpha (n (n.dE) - dE);  H: n x dE + alpha (n (n.dH) - dH), with
       // impedances as in stage_kernel.cuh (the same expressions: the same rounding)
       float fl[6];
-      if (!EXT || !A.mat) {
+      if (!mat) {
         const float v[6] = {
             -(ny * dHz - nz * dHy) + al * (nx * ndE - dEx),
             -(nz * dHx - nx * dHz) + al * (ny * ndE - dEy),
@@ -186,18 +208,19 @@ direct_stage_kernel(const __grid_constant__ StageArgs A, const __grid_constant__
       }
     }
   }
-  float wE = 1.f, wH = 1.f;
-  if (EXT && A.mat) {                              // rhs_E / eps, rhs_H / mu
-    const float4 w = __ldg(A.mat + size_t(k) * kMatVecs);
-    wE = w.x;
-    wH = w.y;
+  if constexpr (EXT == Ext::any) {
+    if (mat) {
+      const float4 w = __ldg(A.mat + size_t(k) * kMatVecs);
+      wE = w.x;
+      wH = w.y;
+    }
   }
   const float dt = RK ? (A.dt_elem ? __ldg(A.dt_elem + k) : A.dt) : 1.f;
 #pragma unroll
   for (int c = 0; c < 6; ++c) {
     float r[Np];
 #pragma unroll
-    for (int i = 0; i < Np; ++i) r[i] = EXT ? rhs[c][i] * (c < 3 ? wE : wH) : rhs[c][i];
+    for (int i = 0; i < Np; ++i) r[i] = EXT != Ext::none ? rhs[c][i] * (c < 3 ? wE : wH) : rhs[c][i];
     const size_t at = size_t(c) * K + k;
     if (RK) {
       const float4 o = reinterpret_cast<const float4*>(A.res)[at];
