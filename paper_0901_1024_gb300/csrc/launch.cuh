@@ -32,9 +32,11 @@ constexpr int kSmSmem = 228 * 1024, kCtaSmem = 1024;
 // contended: a CTA signals its successor before it allocates, so a CTA of the next grid
 // beside it could take the columns and then wait for the grid whose CTA waits for them.
 // A CTA of all 512 columns shares its SM with no other CTA of this size, one of 256 with
-// one more of 256 at most.
+// one more of 256 at most.  The smaller floor is the low one because shared memory is taken
+// from L1, which the neighbour gathers of two CTAs need (order 2 at a floor of 110 KB: 279 936
+// tetrahedra in random order 224 us a stage instead of 141).
 constexpr int tc_smem(int columns, int bytes) {
-  const int least = (columns > 256 ? 120 : 110) * 1024;
+  const int least = (columns > 256 ? 148 : 80) * 1024;
   return bytes > least ? bytes : least;
 }
 static_assert(2 * (tc_smem(256, 0) + kCtaSmem) <= kSmSmem, "two CTAs of 256 columns fit");
