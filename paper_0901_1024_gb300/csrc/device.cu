@@ -380,6 +380,7 @@ struct DeviceState {
   void* tcB = nullptr;          // tensor-core B pieces (orders <= kTcMaxOrder)
   float4* mat = nullptr;        // material records (meshes with materials), in the arena
   bool absorbing = false;       // some boundary face is absorbing
+  bool scattered = false;       // most faces' neighbours lie far off
   float* tcgeo = nullptr;       // word-major geometry for the tensor-core stage
   int tc_geo_stride = 0;
   float tc_inv_bscale = 1.f;
@@ -717,6 +718,7 @@ int ensure_device(dg_mesh* m, std::string& err) {
     }
     std::memcpy(&g[10], &codes, 4);
   }
+  d->scattered = dgdev::scattered_mesh(m->nbr_elem.data(), m->nbr_code.data(), K);
   if (mat_b) {
     // material records: 1/eps, 1/mu, eps, mu, then the flux coefficients of each
     // face from the impedances of both sides (the element's own on boundaries)
@@ -806,6 +808,7 @@ static dgdev::StageArgs stage_args(dg_mesh* m, Path p) {
   a.geo = d->geo;
   a.mat = d->mat;
   a.absorbing = d->absorbing ? 1 : 0;
+  a.scattered = d->scattered ? 1 : 0;
   a.D4 = d->D4;
   a.LIFT4 = d->LIFT4;
   a.fmask = d->fmask;

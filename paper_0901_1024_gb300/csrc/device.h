@@ -54,6 +54,22 @@ __host__ __device__ constexpr int wide_chunk_bytes(int N) {
   return ((d > l ? d : l) + 127) / 128 * 128;
 }
 
+// Whether more than half of a mesh's interior faces have their neighbour over kFarElements
+// elements away in the element order (random order: none near by once the mesh is large).
+// nbr[4 K], code[4 K]: neighbour and its code (< 0: boundary) of each face.
+constexpr int64_t kFarElements = 22000;
+template <class Nbr, class Code>
+bool scattered_mesh(const Nbr* nbr, const Code* code, int64_t K) {
+  int64_t interior = 0, far = 0;
+  for (int64_t i = 0; i < 4 * K; ++i) {
+    if (code[i] < 0) continue;
+    const int64_t d = int64_t(nbr[i]) - i / 4;
+    ++interior;
+    far += d > kFarElements || d < -kFarElements;
+  }
+  return 2 * far > interior;
+}
+
 struct StageArgs {
   const float* u_in;       // [6][K][Np]
   float* u_out;            // [6][K][Np] (RK mode)
@@ -79,6 +95,7 @@ struct StageArgs {
   const void* wide;         // register-tiled FP32 stage: packed operator chunks
   int* status;              // set to 1 if a stage kernel's bounded wait ran out
   int absorbing;            // 1 if any boundary face is absorbing (code kAbsorbingCode)
+  int scattered;            // 1 if most faces' neighbours lie far off (scattered_mesh)
 };
 
 // Tensor-core stage: elements per tile.  Orders <= 4: 6 * 20 = 120 of the 128

@@ -855,9 +855,15 @@ cudaError_t launch_tc_stage_form(bool rk, const StageArgs& a, int num_sms, cudaS
 // of a pair then works alone, at the pace of two (400 tiles 12.7 us
 // against 11.4 in one CTA an SM, 740 17.3 against 16.6, with materials 13.3 and 11.9, 18.3 and
 // 17.3; 360 tiles 11.2 and 11.4, 456 11.3 and 11.5, 680 15.4 and 16.5; from seven rounds on within 1 %).
+// Nor, at order 3, on a mesh in an order that scatters the neighbours (scattered_mesh): the
+// gathers then come from HBM, and two CTAs of 109 KB leave them little L1 (146 334
+// tetrahedra in random order 166 us against 153 in one CTA an SM, 384 000 483 against 413; with
+// half of them moved, 0.54 and 0.67 of the faces far, 149 and 146, 416 and 384; a quarter, 0.32
+// and 0.39, 132 and 140, 353 and 366; shuffled within 40 000, 0.17, 139 and 141).
 // Order 1 on request and order 4 (whose tiles do not fit twice) as one.
-constexpr bool tc_paired(int N, int tiles, int sms) {
+constexpr bool tc_paired(int N, int tiles, int sms, bool scattered) {
   if (N != 3) return N == 2;
+  if (scattered) return false;
   const int rest = tiles % (2 * sms);              // tiles of the last round of CTA pairs
   const bool half = 2 * rest > sms && rest < sms;
   return tiles > sms && !(half && tiles < 5 * sms);
@@ -866,7 +872,7 @@ constexpr bool tc_paired(int N, int tiles, int sms) {
 template <int N>
 cudaError_t launch_tc_stage_n(bool rk, const StageArgs& a, int num_sms, cudaStream_t s) {
   if constexpr (N == 2 || N == 3)
-    if (tc_paired(N, a.num_tiles, num_sms)) return launch_tc_stage_form<N, true>(rk, a, num_sms, s);
+    if (tc_paired(N, a.num_tiles, num_sms, a.scattered)) return launch_tc_stage_form<N, true>(rk, a, num_sms, s);
   if constexpr (N != 2) return launch_tc_stage_form<N, false>(rk, a, num_sms, s);
   return cudaErrorInvalidValue;                    // not reached
 }

@@ -13,6 +13,7 @@ from paper_0901_1024_gb300 import build as b
 
 PROGRAM = r"""
 #include <cstdio>
+#include <vector>
 #include "tc_stage.cuh"
 #include "tc_stage_t.cuh"
 using namespace dgdev;
@@ -35,7 +36,20 @@ int main() {
                 tc_cta_alone(tiles, 152) ? tc_smem(512, TcDims<2, true>::SMEM) : 0);
   for (int N = 1; N <= 4; ++N)
     for (int tiles : {1, 152, 153, 304, 360, 381, 400, 455, 456, 608, 680, 700, 759, 760, 1000, 7317})
-      std::printf("pair%d_%d %d 0\n", N, tiles, tc_paired(N, tiles, 152) ? 1 : 0);
+      std::printf("pair%d_%d %d %d\n", N, tiles, tc_paired(N, tiles, 152, false) ? 1 : 0,
+                  tc_paired(N, tiles, 152, true) ? 1 : 0);
+  // rings of K elements whose neighbours lie `hop` elements on, boundary faces among them
+  for (int K : {1000, 50000})
+    for (int hop : {1, 21999, 22001, 24999}) {
+      std::vector<int32_t> nbr(4 * K);
+      std::vector<signed char> code(4 * K);
+      for (int i = 0; i < 4 * K; ++i) {
+        const int k = i / 4;
+        nbr[i] = (k + (i % 4 < 2 ? hop % K : K - hop % K)) % K;
+        code[i] = i % 4 == 3 ? -1 : 5;
+      }
+      std::printf("far%d_%d %d 0\n", K, hop, scattered_mesh(nbr.data(), code.data(), K) ? 1 : 0);
+    }
 }
 """
 
@@ -81,3 +95,15 @@ def test_which_launches_are_paired(forms):
         assert [forms[f"pair{N}_{tiles}"][0] for N in (1, 2, 4)] == [0, 1, 0]
         single = tiles <= 152 or 380 < tiles < 456 or 684 < tiles < 760
         assert forms[f"pair3_{tiles}"][0] == (0 if single else 1), tiles
+        # a mesh whose neighbours are scattered: order 3 never
+        assert [forms[f"pair{N}_{tiles}"][1] for N in (1, 2, 3, 4)] == [0, 1, 0, 0]
+
+
+def test_which_meshes_are_scattered(forms):
+    """Faces over 22 000 elements away count; rings wrap, so a hop h is h or K - h away."""
+    for K in (1000, 50000):
+        for hop in (1, 21999, 22001, 24999):
+            h = hop % K
+            away = [h] * (K - h) + [K - h] * h              # forward; backward alike
+            far = sum(a > 22000 for a in away)
+            assert forms[f"far{K}_{hop}"][0] == int(2 * far > K), (K, hop)
