@@ -25,7 +25,6 @@ __device__ __forceinline__ int mixed_group(const MixedArgs& M) {
 }
 
 __global__ void __launch_bounds__(640, 1) tc_mixed_kernel(const __grid_constant__ MixedArgs M) {
-  pdl_launch_dependents();
   const MixedGroup& g = M.g[mixed_group(M)];
   const int cta = int(blockIdx.x) - g.first;
   switch (g.N * 2 + g.ext) {

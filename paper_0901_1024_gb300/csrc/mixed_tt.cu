@@ -13,6 +13,7 @@ namespace {
 
 constexpr int kMixedTtSmem = tc_smem(512, TtDims<5>::SMEM > TtDims<6>::SMEM ? TtDims<5>::SMEM
                                                                              : TtDims<6>::SMEM);
+static_assert(tc_sole(kMixedTtSmem), "signals before it has its columns");
 static_assert(TtDims<5>::THREADS == TtDims<6>::THREADS, "one CTA shape");
 
 __global__ void __launch_bounds__(TtDims<6>::THREADS, 1)

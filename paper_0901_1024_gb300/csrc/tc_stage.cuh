@@ -534,7 +534,10 @@ __device__ __forceinline__ void tc_stage_body(const StageArgs& A, const int cta,
   // ---- set-up: B pieces (one bulk copy, constant data: it may overlap the
   // previous kernel), face-node table, tensor memory, barriers ----------------
   for (int i = tid; i < 4 * Nfp; i += D::THREADS) sFmask[i] = __ldg(A.fmask + i);
-  if (warp == 0) tc::tmem_alloc(&s_tmem, D::TMEM);
+  if (warp == 0) {
+    tc::tmem_alloc(&s_tmem, D::TMEM);
+    pdl_launch_dependents();                       // not before: tc_smem()
+  }
   if (tid == 0) {
     tc::mbar_init(&s_b_full, 1);
     for (int i = 0; i < D::NSU; ++i) tc::mbar_init(&s_u_full[i], 1);
@@ -811,7 +814,6 @@ __device__ __forceinline__ void tc_stage_body(const StageArgs& A, const int cta,
 template <int N, bool RK, bool EXT, bool PAIR>
 __global__ void __launch_bounds__(TcDims<N, PAIR>::THREADS, PAIR ? 2 : 1)
 tc_stage_kernel(const __grid_constant__ StageArgs A) {
-  pdl_launch_dependents();
   tc_stage_body<N, RK, EXT, PAIR>(A, int(blockIdx.x), int(gridDim.x));
 }
 
@@ -857,7 +859,7 @@ cudaError_t launch_tc_stage_form(bool rk, const StageArgs& a, int num_sms, cudaS
 // 17.3; 360 tiles 11.2 and 11.4, 456 11.3 and 11.5, 680 15.4 and 16.5; from seven rounds on within 1 %).
 // Nor, at order 3, on a mesh in an order that scatters the neighbours (scattered_mesh): the
 // gathers then come from HBM, and two CTAs of 109 KB leave them little L1 (146 334
-// tetrahedra in random order 166 us against 153 in one CTA an SM, 384 000 483 against 413; with
+// tetrahedra in random order 166 us against 151 in one CTA an SM, 384 000 483 against 400; with
 // half of them moved, 0.54 and 0.67 of the faces far, 149 and 146, 416 and 384; a quarter, 0.32
 // and 0.39, 132 and 140, 353 and 366; shuffled within 40 000, 0.17, 139 and 141).
 // Order 1 on request and order 4 (whose tiles do not fit twice) as one.

@@ -764,6 +764,7 @@ cudaError_t launch_tt_stage_n(bool rk, const StageArgs& a, int num_sms, cudaStre
   auto kern = rk ? (ext ? tt_stage_kernel<N, true, true> : tt_stage_kernel<N, true, false>)
                  : (ext ? tt_stage_kernel<N, false, true> : tt_stage_kernel<N, false, false>);
   constexpr int smem = tc_smem(512, D::SMEM);
+  static_assert(tc_sole(smem), "signals before it has its columns");
   bool& done = attr[rk ? 1 : 0][ext ? 1 : 0][dev];
   if (!done) {
     err = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, smem);
