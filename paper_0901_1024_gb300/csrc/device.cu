@@ -380,7 +380,7 @@ struct DeviceState {
   void* tcB = nullptr;          // tensor-core B pieces (orders <= kTcMaxOrder)
   float4* mat = nullptr;        // material records (meshes with materials), in the arena
   bool absorbing = false;       // some boundary face is absorbing
-  bool scattered = false;       // most faces' neighbours lie far off
+  bool scattered = false;       // most faces' neighbours lie far off (order 3: tc_paired)
   float* tcgeo = nullptr;       // word-major geometry for the tensor-core stage
   int tc_geo_stride = 0;
   float tc_inv_bscale = 1.f;
@@ -718,7 +718,7 @@ int ensure_device(dg_mesh* m, std::string& err) {
     }
     std::memcpy(&g[10], &codes, 4);
   }
-  d->scattered = dgdev::scattered_mesh(m->nbr_elem.data(), m->nbr_code.data(), K);
+  d->scattered = m->N == 3 && dgdev::scattered_mesh(m->nbr_elem.data(), m->nbr_code.data(), K);
   if (mat_b) {
     // material records: 1/eps, 1/mu, eps, mu, then the flux coefficients of each
     // face from the impedances of both sides (the element's own on boundaries)

@@ -55,18 +55,20 @@ __host__ __device__ constexpr int wide_chunk_bytes(int N) {
 }
 
 // Whether more than half of a mesh's interior faces have their neighbour over kFarElements
-// elements away in the element order (random order: none near by once the mesh is large).
+// elements away in the element order (random order: none near by once the mesh is large),
+// looking at every (1 + K / 8 192)th element (all faces of 705 894 took 2.5 ms).
 // nbr[4 K], code[4 K]: neighbour and its code (< 0: boundary) of each face.
 constexpr int64_t kFarElements = 22000;
 template <class Nbr, class Code>
 bool scattered_mesh(const Nbr* nbr, const Code* code, int64_t K) {
   int64_t interior = 0, far = 0;
-  for (int64_t i = 0; i < 4 * K; ++i) {
-    if (code[i] < 0) continue;
-    const int64_t d = int64_t(nbr[i]) - i / 4;
-    ++interior;
-    far += d > kFarElements || d < -kFarElements;
-  }
+  for (int64_t k = 0, step = 1 + K / 8192; k < K; k += step)
+    for (int64_t i = 4 * k; i < 4 * k + 4; ++i) {
+      if (code[i] < 0) continue;
+      const int64_t d = int64_t(nbr[i]) - k;
+      ++interior;
+      far += d > kFarElements || d < -kFarElements;
+    }
   return 2 * far > interior;
 }
 
