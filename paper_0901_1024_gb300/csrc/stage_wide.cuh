@@ -306,6 +306,10 @@ __global__ void __launch_bounds__(WideDims<N>::T, 1) stage_wide_kernel(const __g
     }
     __syncthreads();
   }
+  // every chunk has been waited for; after a wait that ran out, once more (as bounded) for
+  // the last copy into each buffer before the shared memory is given up
+  if (tid == 0)
+    for (int i = max(n - 2, 0); i < n; ++i) wait_or_flag(&s_full[i & 1], (i >> 1) & 1, A.status);
 }
 
 template <int N>
